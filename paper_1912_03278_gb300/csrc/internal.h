@@ -84,6 +84,10 @@ cudaError_t launch_fused_lattice(const FusedArgs &a, const Schedule &sched, int 
 // dst <- src, bytes a multiple of 16 and both 16-byte aligned, by a grid-stride
 // kernel (src may be pinned host memory the device can address)
 cudaError_t launch_copy16(const void *src, void *dst, size_t bytes, cudaStream_t s);
+// out (device memory of this GPU, 4-byte aligned, n_chains * N floats) <- the
+// chains' current configurations
+cudaError_t launch_gather_chains(float *const psi[3], const ChainState *st, float *out, int64_t N,
+                                 int n_chains, cudaStream_t s);
 // start = prop = 0 in every chain's state (a configuration was set from outside)
 cudaError_t launch_reset_chain_start(ChainState *st, int n, cudaStream_t s);
 int fused_lattice_smem_bytes(const Geometry &g, int depth, int vec);

@@ -1249,15 +1249,37 @@ ising_status ising_hmc_chain_params(const ising_hmc_t *h, double *out) {
 
 ising_status ising_hmc_get_state_native(ising_hmc_t *h, void *out) {
     if (!h || !out) return ISING_EINVAL;
+    const size_t cb = (size_t)h->N * state_elem(h);
+    if (!is_fused(h)) {   // one buffer holds every chain
+        ising_status st = ising_hmc_sync(h);
+        if (st != ISING_OK) return st;
+        CUDA_OR_FAIL(h, cudaMemcpyAsync(out, h->psi[0], cb * h->n_chains, cudaMemcpyDefault, h->stream));
+        CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
+        return ISING_OK;
+    }
+    // memory of the GPU the handle's buffers are on: one gather launch;
+    // anything else (host memory, another GPU) chain by chain
+    cudaPointerAttributes pa{}, pm{};
+    const bool local = cudaPointerGetAttributes(&pa, out) == cudaSuccess &&
+                       cudaPointerGetAttributes(&pm, h->psi[0]) == cudaSuccess &&
+                       pa.type == cudaMemoryTypeDevice && pm.type == cudaMemoryTypeDevice &&
+                       pa.device == pm.device && (uintptr_t)out % sizeof(float) == 0;
+    cudaGetLastError();
+    if (local) {
+        ising_status st = ising_hmc_sync(h);
+        if (st != ISING_OK) return st;
+        float *const psi[3] = {(float *)h->psi[0], (float *)h->psi[1], (float *)h->psi[2]};
+        CUDA_OR_FAIL(h, launch_gather_chains(psi, h->d_state, (float *)out, h->N, h->n_chains, h->stream));
+        h->launches += 1;
+        CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
+        return ISING_OK;
+    }
     std::vector<ChainState> hs;
     ising_status st = fetch_states(h, hs);
     if (st != ISING_OK) return st;
-    const size_t cb = (size_t)h->N * state_elem(h);
-    for (int c = 0; c < h->n_chains; ++c) {
-        const int b = is_fused(h) ? hs[c].start : 0;
-        CUDA_OR_FAIL(h, cudaMemcpyAsync((char *)out + c * cb, (const char *)h->psi[b] + c * cb, cb,
-                                        cudaMemcpyDefault, h->stream));
-    }
+    for (int c = 0; c < h->n_chains; ++c)
+        CUDA_OR_FAIL(h, cudaMemcpyAsync((char *)out + c * cb, (const char *)h->psi[hs[c].start] + c * cb,
+                                        cb, cudaMemcpyDefault, h->stream));
     CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
     return ISING_OK;
 }
