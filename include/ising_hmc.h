@@ -230,7 +230,15 @@ int64_t ising_hmc_launch_count(const ising_hmc_t *h);
 /* Synchronise the handle's stream; ETIMEOUT if a device wait gave up. */
 ising_status ising_hmc_sync(ising_hmc_t *h);
 
-/* Launch shape of the fused FP32 lattice kernel: threads per CTA (a multiple
+/* 2D lattices (rows of at most 1024 sites, at least 24 rows) whose launch shape
+ * and plane staging were left to the library and whose chains are not split run
+ * on a kernel that marches down the rows and takes several force evaluations
+ * per sweep; it has no shape to choose.  Its psi and p are bit for bit those of
+ * the plane-streaming kernel below, which a call of ising_hmc_set_launch,
+ * ising_hmc_set_chain_split or ising_hmc_set_staging selects; the FP64 sums
+ * (action, energies, estimators) equal them to rounding.
+ *
+ * Launch shape of the fused FP32 lattice kernel: threads per CTA (a multiple
  * of 32, at most 4 float4 vectors of a plane per thread; 32..256 with one CTA
  * per chain, up to 512 when chains are split over CTAs, see
  * ising_hmc_set_chain_split) and the prefetch depth in planes (1, 2 or 4; the
@@ -257,7 +265,8 @@ int ising_hmc_get_chain_split(const ising_hmc_t *h);
  * with cp.async; ISING_STAGING_BULK, one lane issues each plane as a bulk
  * copy completing on an mbarrier (planes of whole 16-byte vectors: rows of a
  * multiple of 4 sites); ISING_STAGING_AUTO (default), bulk for planes of at
- * least 4 KB.  Results are bit for bit the same in every mode.  EINVAL for
+ * least 4 KB.  Results are bit for bit the same in both modes, and psi and p
+ * under the automatic choice as well.  EINVAL for
  * other forms, unknown modes, or bulk on rows that are not a multiple of 4. */
 enum { ISING_STAGING_AUTO = 0, ISING_STAGING_THREADS = 1, ISING_STAGING_BULK = 2 };
 ising_status ising_hmc_set_staging(ising_hmc_t *h, int mode);

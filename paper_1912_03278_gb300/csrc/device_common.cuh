@@ -85,6 +85,59 @@ __device__ __forceinline__ float4 spin_u4_f32(uint32_t q, uint32_t traj, uint32_
     const u32x4 x = philox(q, traj, chain, PURPOSE_SPIN, seed);
     return make_float4(u23(x.x), u23(x.y), u23(x.z), u23(x.w));
 }
+// The same draws with the key schedule given (round r's keys rk[2r], rk[2r+1]):
+// where it comes from the kernel's constant parameters, a round costs no
+// integer additions.
+__device__ __forceinline__ u32x4 philox(uint32_t idx, uint32_t traj, uint32_t chain,
+                                        uint32_t purpose, const uint32_t *rk) {
+    uint32_t c0 = idx, c1 = traj, c2 = chain, c3 = purpose;
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const uint64_t m0 = (uint64_t)0xD2511F53u * c0, m1 = (uint64_t)0xCD9E8D57u * c2;
+        const uint32_t n0 = (uint32_t)(m1 >> 32) ^ c1 ^ rk[2 * r];
+        const uint32_t n2 = (uint32_t)(m0 >> 32) ^ c3 ^ rk[2 * r + 1];
+        c0 = n0;
+        c1 = (uint32_t)m1;
+        c2 = n2;
+        c3 = (uint32_t)m0;
+    }
+    return u32x4{c0, c1, c2, c3};
+}
+__device__ __forceinline__ float4 momenta4(uint32_t q, uint32_t traj, uint32_t chain,
+                                           const uint32_t *rk) {
+    const u32x4 x = philox(q, traj, chain, PURPOSE_MOM, rk);
+    float4 z;
+    box_muller_f32(u23(x.x), u23(x.y), z.x, z.y);
+    box_muller_f32(u23(x.z), u23(x.w), z.z, z.w);
+    return z;
+}
+__device__ __forceinline__ float4 spin_u4(uint32_t q, uint32_t traj, uint32_t chain,
+                                          const uint32_t *rk) {
+    const u32x4 x = philox(q, traj, chain, PURPOSE_SPIN, rk);
+    return make_float4(u23(x.x), u23(x.y), u23(x.z), u23(x.w));
+}
+// For the four sites site0 .. site0 + 3 when site0 is not a multiple of 4: two
+// random blocks, the four values from both.
+__device__ __forceinline__ void four_of_eight(const float4 &a, const float4 &b, uint32_t off, float (&z)[4]) {
+    z[0] = off == 0 ? a.x : off == 1 ? a.y : off == 2 ? a.z : a.w;
+    z[1] = off == 0 ? a.y : off == 1 ? a.z : off == 2 ? a.w : b.x;
+    z[2] = off == 0 ? a.z : off == 1 ? a.w : off == 2 ? b.x : b.y;
+    z[3] = off == 0 ? a.w : off == 1 ? b.x : off == 2 ? b.y : b.z;
+}
+__device__ __forceinline__ void momenta4_any(uint32_t site0, uint32_t traj, uint32_t chain,
+                                             const uint32_t *rk, float (&z)[4]) {
+    const uint32_t off = site0 & 3;
+    const float4 a = momenta4(site0 >> 2, traj, chain, rk);
+    const float4 b = off ? momenta4((site0 >> 2) + 1, traj, chain, rk) : a;
+    four_of_eight(a, b, off, z);
+}
+__device__ __forceinline__ void spin_u4_any(uint32_t site0, uint32_t traj, uint32_t chain,
+                                            const uint32_t *rk, float (&u)[4]) {
+    const uint32_t off = site0 & 3;
+    const float4 a = spin_u4(site0 >> 2, traj, chain, rk);
+    const float4 b = off ? spin_u4((site0 >> 2) + 1, traj, chain, rk) : a;
+    four_of_eight(a, b, off, u);
+}
 // Two FP64 momenta for sites 2*q, 2*q+1 (FP64 form).
 __device__ __forceinline__ void momenta2_f64(uint32_t q, uint32_t traj, uint32_t chain,
                                              uint64_t seed, double &z0, double &z1) {

@@ -178,15 +178,14 @@ struct Slots {
 };
 
 template <int VEC>
-__device__ __forceinline__ Slots make_slots(const Geometry &g) {
+__device__ __forceinline__ Slots make_slots(const Geometry &g, int tid, int nt) {
     Slots s;
     const int nvec = g.P / VEC;
-    const int nt = blockDim.x;
-    const int wbase = threadIdx.x & ~31;
+    const int wbase = tid & ~31;
     s.nwarp = 0;
 #pragma unroll
     for (int k = 0; k < NVMAX; ++k) {
-        const int v = threadIdx.x + k * nt;
+        const int v = tid + k * nt;
         s.valid[k] = v < nvec;
         const int vc = v < nvec ? v : nvec - 1;
         s.e0[k] = vc * VEC;
@@ -745,6 +744,98 @@ __device__ __forceinline__ void set_obs(ChainState *st, const ChainParams &prm, 
     st->obs[3] = fabs(m);
 }
 
+// The threads of one CTA's share of a chain as the steps below see them: the
+// one that keeps the chain's state, and a barrier.
+struct CtaThreads {
+    __device__ __forceinline__ bool first() const { return threadIdx.x == 0; }
+    __device__ __forceinline__ void sync() const { __syncthreads(); }
+};
+
+// Metropolis decision of trajectory traj (Sec. 3) from the chain totals v =
+// {K0, K1, S1, sum t, sum a.t, sum h'.t, sum of spins} of the proposal in
+// buffer prop.  S_cur (thread 0 of every CTA of the chain): the action of the
+// current configuration; lead: this CTA writes the chain's state.  Returns the
+// buffer of the current configuration afterwards, in every thread.
+template <class Threads>
+__device__ __forceinline__ int metropolis_step(const Threads &th, const FusedArgs &A, ChainState *st,
+                                               const ChainParams &prm, int chain, uint32_t traj,
+                                               int start, int prop, const double (&v)[7],
+                                               double invN, double &S_cur, bool lead, int *bcast) {
+    if (th.first()) {
+        const double S0 = S_cur;
+        const double dH = (v[1] + v[2]) - (v[0] + S0);
+        const double logu = accept_logu(traj, (uint32_t)chain, A.seed, PURPOSE_ACC);
+        const bool accd = logu < -dH;
+        if (lead) {
+            st->prop = prop;
+            st->rec[ISING_REC_DH] = dH;
+            st->rec[ISING_REC_LOGU] = logu;
+            st->rec[ISING_REC_ACCEPTED] = accd ? 1.0 : 0.0;
+            st->rec[ISING_REC_K0] = v[0];
+            st->rec[ISING_REC_S0] = S0;
+            st->rec[ISING_REC_K1] = v[1];
+            st->rec[ISING_REC_S1] = v[2];
+            st->rec[ISING_REC_FLIPPED] = 0.0;
+            if (accd) {
+                st->start = prop;
+                st->S = v[2];
+                set_obs(st, prm, v[3], v[4], v[5], v[6], invN);
+            }
+        }
+        if (accd) S_cur = v[2];
+        bcast[0] = accd ? prop : start;
+    }
+    th.sync();
+    const int cur = bcast[0];
+    th.sync();
+    return cur;
+}
+
+// Metropolis decision of the global sign flip (Sec. 3) from the totals w =
+// {S(-psi), sum t, sum a.t, sum h'.t, sum of spins}; every thread learns it.
+template <class Threads>
+__device__ __forceinline__ bool flip_step(const Threads &th, const FusedArgs &A, ChainState *st, const ChainParams &prm,
+                                          int chain, uint32_t traj, const double (&w)[5],
+                                          double invN, double &S_cur, bool lead, int *bcast) {
+    if (th.first()) {
+        const double lu = accept_logu(traj, (uint32_t)chain, A.seed, PURPOSE_FLIP);
+        const bool fl = lu < -(w[0] - S_cur);
+        if (fl) {
+            S_cur = w[0];
+            if (lead) {
+                st->S = w[0];
+                set_obs(st, prm, w[1], w[2], w[3], w[4], invN);
+                st->rec[ISING_REC_FLIPPED] = 1.0;
+            }
+        }
+        bcast[1] = fl ? 1 : 0;
+    }
+    th.sync();
+    return bcast[1] != 0;
+}
+
+// Adds the trajectory's measurement to the chain's sums (a repeated
+// configuration repeats its measurement).
+template <class Threads>
+__device__ __forceinline__ void measure_step(const Threads &th, const FusedArgs &A, ChainState *st, uint32_t traj,
+                                             bool lead) {
+    if (th.first() && lead && (int64_t)traj >= (int64_t)A.n_therm) {
+        double *sm = st->sums;
+        const double dH = st->rec[ISING_REC_DH];
+        sm[ISING_SUM_NMEAS] += 1.0;
+        sm[ISING_SUM_NACC] += st->rec[ISING_REC_ACCEPTED];
+        sm[ISING_SUM_M] += st->obs[0];
+        sm[ISING_SUM_M2] += st->obs[0] * st->obs[0];
+        sm[ISING_SUM_E] += st->obs[1];
+        sm[ISING_SUM_E2] += st->obs[1] * st->obs[1];
+        sm[ISING_SUM_ABSM] += st->obs[2];
+        sm[ISING_SUM_ABSM2] += st->obs[2] * st->obs[2];
+        sm[ISING_SUM_DH] += dH;
+        sm[ISING_SUM_EXPMDH] += exp(-dH);
+    }
+    th.sync();
+}
+
 // CL: compiled for chains split over a cluster (launched with a cluster
 // size); the unsplit instance carries no cluster instructions at all.
 template <int DIM, int VEC, int D, bool CL, bool BULK>
@@ -779,7 +870,7 @@ __global__ void __launch_bounds__(CL ? MAX_THREADS : MAX_THREADS_UNSPLIT, CL ? 1
     ChainState *st = A.state + chain;
     const ChainParams prm = A.params[chain];
     const double invN = 1.0 / (double)g.N;
-    const Slots sl = make_slots<VEC>(g);
+    const Slots sl = make_slots<VEC>(g, threadIdx.x, blockDim.x);
 
     if (A.mode == MODE_MOMENTA) {
         momenta_sweep<VEC>(A, chain, A.traj0, sl, z0, z1);
@@ -871,33 +962,7 @@ __global__ void __launch_bounds__(CL ? MAX_THREADS : MAX_THREADS_UNSPLIT, CL ? 1
                        acc_val(acc.S, acc.Slo), kahan_val(acc.sT, acc.cT),
                        kahan_val(acc.sAT, acc.cAT), kahan_val(acc.sHT, acc.cHT), (double)acc.sS};
         chain_sum<7, CL>(v, red, xch, cs);
-        if (threadIdx.x == 0) {
-            const double S0 = S_cur;
-            const double dH = (v[1] + v[2]) - (v[0] + S0);
-            const double logu = accept_logu(traj, (uint32_t)chain, A.seed, PURPOSE_ACC);
-            const bool accd = logu < -dH;
-            if (lead) {
-                st->prop = prop;
-                st->rec[ISING_REC_DH] = dH;
-                st->rec[ISING_REC_LOGU] = logu;
-                st->rec[ISING_REC_ACCEPTED] = accd ? 1.0 : 0.0;
-                st->rec[ISING_REC_K0] = v[0];
-                st->rec[ISING_REC_S0] = S0;
-                st->rec[ISING_REC_K1] = v[1];
-                st->rec[ISING_REC_S1] = v[2];
-                st->rec[ISING_REC_FLIPPED] = 0.0;
-                if (accd) {
-                    st->start = prop;
-                    st->S = v[2];
-                    set_obs(st, prm, v[3], v[4], v[5], v[6], invN);
-                }
-            }
-            if (accd) S_cur = v[2];
-            bcast[0] = accd ? prop : start;
-        }
-        __syncthreads();
-        start = bcast[0];
-        __syncthreads();
+        start = metropolis_step(CtaThreads{}, A, st, prm, chain, traj, start, prop, v, invN, S_cur, lead, bcast);
         // ---- optional global sign flip psi -> -psi (Sec. 3, ergodicity) ----
         if (A.flip_every > 0 && ((traj + 1) % (uint32_t)A.flip_every) == 0) {
             Acc fa = acc_zero();
@@ -905,21 +970,7 @@ __global__ void __launch_bounds__(CL ? MAX_THREADS : MAX_THREADS_UNSPLIT, CL ? 1
             double w[5] = {acc_val(fa.S, fa.Slo), kahan_val(fa.sT, fa.cT),
                            kahan_val(fa.sAT, fa.cAT), kahan_val(fa.sHT, fa.cHT), (double)fa.sS};
             chain_sum<5, CL>(w, red, xch + XCH_WORDS, cs);
-            if (threadIdx.x == 0) {
-                const double lu = accept_logu(traj, (uint32_t)chain, A.seed, PURPOSE_FLIP);
-                const bool fl = lu < -(w[0] - S_cur);
-                if (fl) {
-                    S_cur = w[0];
-                    if (lead) {
-                        st->S = w[0];
-                        set_obs(st, prm, w[1], w[2], w[3], w[4], invN);
-                        st->rec[ISING_REC_FLIPPED] = 1.0;
-                    }
-                }
-                bcast[1] = fl ? 1 : 0;
-            }
-            __syncthreads();
-            if (bcast[1]) {
+            if (flip_step(CtaThreads{}, A, st, prm, chain, traj, w, invN, S_cur, lead, bcast)) {
                 // -psi goes to the buffer that is neither current nor the proposal,
                 // so the MD end point stays readable
                 const int f = (start != prop) ? 3 - start - prop : (start + 1) % 3;
@@ -936,41 +987,26 @@ __global__ void __launch_bounds__(CL ? MAX_THREADS : MAX_THREADS_UNSPLIT, CL ? 1
             __syncthreads();
         }
         // ---- measurement: a repeated configuration repeats its measurement ----
-        if (threadIdx.x == 0 && lead && (int64_t)traj >= (int64_t)A.n_therm) {
-            double *sm = st->sums;
-            const double dH = st->rec[ISING_REC_DH];
-            sm[ISING_SUM_NMEAS] += 1.0;
-            sm[ISING_SUM_NACC] += st->rec[ISING_REC_ACCEPTED];
-            sm[ISING_SUM_M] += st->obs[0];
-            sm[ISING_SUM_M2] += st->obs[0] * st->obs[0];
-            sm[ISING_SUM_E] += st->obs[1];
-            sm[ISING_SUM_E2] += st->obs[1] * st->obs[1];
-            sm[ISING_SUM_ABSM] += st->obs[2];
-            sm[ISING_SUM_ABSM2] += st->obs[2] * st->obs[2];
-            sm[ISING_SUM_DH] += dH;
-            sm[ISING_SUM_EXPMDH] += exp(-dH);
-        }
-        __syncthreads();
+        measure_step(CtaThreads{}, A, st, traj, lead);
     }
     if (CL && cs > 1) cluster_barrier();   // no CTA leaves while its exchange buffers may be read
 }
 
-// Shared-memory size of a launch: with the table if that leaves as many CTAs
-// resident per SM as without it (the occupancy calculator decides), else
-// without.  The last answers are cached per thread.
+// Shared-memory size of a launch that needs `base` bytes: with the table if
+// that leaves as many CTAs resident per SM as without it (the occupancy
+// calculator decides), else without.  The last answers are cached per thread.
 template <class K>
-static int launch_smem(K kern, const Geometry &g, int D, int threads) {
+static int smem_with_table(K kern, int base, int threads) {
     struct Memo {
         const void *kern;
-        int P, D, threads, smem;
+        int base, threads, smem;
     };
     thread_local Memo memo[8] = {};
     thread_local int next = 0;
     for (const Memo &m : memo)
-        if (m.smem && m.kern == reinterpret_cast<const void *>(kern) && m.P == g.P && m.D == D &&
+        if (m.smem && m.kern == reinterpret_cast<const void *>(kern) && m.base == base &&
             m.threads == threads)
             return m.smem;
-    const int base = (int)(ring_bytes(g.P, D) + RED_BYTES);
     const int with_tab = base + LOG1PEXP_NODES * 16;
     int n_with = 0, n_without = 0;
     int smem = base;
@@ -980,7 +1016,7 @@ static int launch_smem(K kern, const Geometry &g, int D, int threads) {
         n_with >= n_without)
         smem = with_tab;
     cudaGetLastError();
-    memo[next] = Memo{reinterpret_cast<const void *>(kern), g.P, D, threads, smem};
+    memo[next] = Memo{reinterpret_cast<const void *>(kern), base, threads, smem};
     next = (next + 1) % 8;
     return smem;
 }
@@ -995,7 +1031,7 @@ cudaError_t kernel_node(const FusedArgs &a, int threads, cudaKernelNodeParams *n
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    const int smem = launch_smem(kern, a.g, D, threads);
+    const int smem = smem_with_table(kern, (int)(ring_bytes(a.g.P, D) + RED_BYTES), threads);
     np->func = reinterpret_cast<void *>(kern);
     np->gridDim = dim3((unsigned)((a.n_chains - a.chain0) * a.cs), 1, 1);
     np->blockDim = dim3((unsigned)threads, 1, 1);

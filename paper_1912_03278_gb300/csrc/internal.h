@@ -55,7 +55,8 @@ struct FusedArgs {
     const ChainParams *params;
     ChainState *state;
     Geometry g;
-    uint64_t seed;
+    uint64_t seed;           // (set by set_seed, with its key schedule)
+    uint32_t round_keys[20], round_keys0[20];   // Philox round keys of seed and of key 0
     uint32_t traj0;          // index of the first trajectory of this launch
     int n_traj;              // trajectories per chain in this launch
     int n_therm;             // trajectories with index < n_therm are not measured
@@ -67,10 +68,23 @@ struct FusedArgs {
     int eval_start;          // lattice kernel: evaluate S and the observables of the start
                              // configuration in the first trajectory's first pass
     int bulk;                // lattice kernel: stage planes by bulk copies (16-byte planes)
+    int march;               // threads per slab of the marching kernel (0: another kernel)
     int *err;
 };
 
 enum { MODE_TRAJ = 0, MODE_EVAL = 1, MODE_MOMENTA = 2 };
+
+// The seed of a launch and the Philox key schedules (Weyl sequences) of it and
+// of key 0, which draws the measurement of a configuration set from outside.
+inline void set_seed(FusedArgs &a, uint64_t seed) {
+    a.seed = seed;
+    for (uint32_t r = 0; r < 10; ++r) {
+        a.round_keys0[2 * r] = r * 0x9E3779B9u;
+        a.round_keys0[2 * r + 1] = r * 0xBB67AE85u;
+        a.round_keys[2 * r] = (uint32_t)seed + a.round_keys0[2 * r];
+        a.round_keys[2 * r + 1] = (uint32_t)(seed >> 32) + a.round_keys0[2 * r + 1];
+    }
+}
 
 // Trajectory index of the spin draw that measures a configuration set from
 // outside (creation, set_state); drawn under key 0.
@@ -99,6 +113,11 @@ cudaError_t fused_lattice_node(const FusedArgs &a, int threads, int depth,
 int fused_lattice_valid_launch(const Geometry &g, int threads, int depth);
 // 1 if a chain may be split over cs CTAs (a thread-block cluster) at that shape.
 int fused_lattice_valid_split(const Geometry &g, int threads, int depth, int cs);
+// Marching kernel (2D, one CTA per chain, several force evaluations per sweep):
+// threads per chain for this geometry (0 if it does not take it); its
+// kernel-node parameters.
+int march_lattice_threads(const Geometry &g);
+cudaError_t march_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args);
 // Cluster size of a graph kernel node made from fused_lattice_node (cs > 1).
 cudaError_t fused_lattice_node_cluster(cudaGraphNode_t node, int cs);
 int fused_lattice_pick(const Geometry &g, int *threads, int *depth);

@@ -44,6 +44,9 @@ struct ising_hmc {
     int *d_err = nullptr;
     // launch shape of the fused kernel: threads per CTA, prefetch depth, CTAs per chain
     int threads = 0, depth = 0, cs = 1, staging = ISING_STAGING_AUTO;
+    // no launch shape asked for: the library may run trajectories on the
+    // marching kernel, which has one shape per lattice
+    bool auto_shape = true;
     // FP32 lattice form: the configurations were set from outside and their
     // action is evaluated by the next trajectory's first force pass
     bool eval_pending = false;
@@ -373,6 +376,16 @@ static int staging_bulk(const ising_hmc *h) {
     if (h->staging == ISING_STAGING_THREADS) return 0;
     return (int64_t)g.P * 4 >= BULK_AUTO_MIN_BYTES;
 }
+
+// Trajectories on the marching kernel: 2D chains on one CTA each, unless a
+// launch shape or a plane staging (choices of the plane-streaming kernel) was
+// asked for.  The kernel's threads per chain, 0 for the other kernels.
+static int use_march(const ising_hmc *h) {
+    const bool may = is_fp32_lattice(h) && h->auto_shape && h->cs == 1 && h->staging == ISING_STAGING_AUTO;
+    return may ? march_lattice_threads(h->g) : 0;
+}
+// What of a handle, besides its shape and split, selects the kernel.
+static int kernel_choice(const ising_hmc *h) { return staging_bulk(h) | (use_march(h) ? 2 : 0); }
 static FusedArgs fused_args(ising_hmc *h) {
     FusedArgs a{};
     for (int i = 0; i < 3; ++i) a.psi[i] = (float *)h->psi[i];
@@ -388,6 +401,7 @@ static FusedArgs fused_args(ising_hmc *h) {
     a.n_chains = h->n_chains;
     a.cs = is_fp32_lattice(h) ? h->cs : 1;
     a.bulk = staging_bulk(h);
+    a.march = use_march(h);
     a.err = h->d_err;
     return a;
 }
@@ -401,7 +415,7 @@ static ising_status eval_current(ising_hmc *h) {
     if (is_fused(h)) {
         FusedArgs a = fused_args(h);
         a.mode = MODE_EVAL;
-        a.seed = 0;
+        set_seed(a, 0);
         a.traj0 = TRAJ_INIT_INDEX;
         a.n_traj = 0;
         CUDA_OR_FAIL(h, launch_fused(h, a));
@@ -1001,7 +1015,7 @@ static ising_status run_trajectories(ising_hmc *h, int64_t n, uint64_t seed) {
             const int64_t k = std::min(per, n - done);
             FusedArgs a = fused_args(h);
             a.mode = MODE_TRAJ;
-            a.seed = seed;
+            set_seed(a, seed);
             a.traj0 = (uint32_t)(h->traj + done);
             a.n_traj = (int)k;
             a.eval_start = done == 0 && h->eval_pending;
@@ -1210,7 +1224,7 @@ ising_status ising_hmc_momenta(ising_hmc_t *h, uint64_t seed, int64_t traj, int 
     } else if (is_fused(h)) {
         FusedArgs a = fused_args(h);
         a.mode = MODE_MOMENTA;
-        a.seed = seed;
+        set_seed(a, seed);
         a.traj0 = (uint32_t)traj;
         a.chain0 = chain0;
         a.n_chains = chain0 + count;
@@ -1338,6 +1352,7 @@ ising_status ising_hmc_set_launch(ising_hmc_t *h, int threads, int depth) {
                     threads, depth, h->cs);
     h->threads = threads;
     h->depth = depth;
+    h->auto_shape = false;
     return ISING_OK;
 }
 
@@ -1419,6 +1434,7 @@ static ising_status clone_for_tuning(ising_hmc *h, int nt, ising_hmc **out) {
         (*out)->depth = h->depth;
         (*out)->cs = h->cs;
         (*out)->staging = h->staging;
+        (*out)->auto_shape = h->auto_shape;
     }
     return st;
 }
@@ -1455,7 +1471,9 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int nt = std::min(h->n_chains, std::max(1, 2 * nsm));
+    // (more of short chains: several CTAs of few warps share an SM)
+    const int64_t most = std::min<int64_t>(8 * nsm, ((int64_t)1 << 28) / h->N);
+    const int nt = (int)std::min<int64_t>(h->n_chains, std::max<int64_t>(std::max(1, 2 * nsm), most));
     ising_hmc *t = nullptr;
     st = clone_for_tuning(h, nt, &t);
     if (st != ISING_OK) return fail(h, st, "autotune: %s", ising_hmc_last_create_error());
@@ -1468,6 +1486,7 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
     const int cand_d[] = {1, 2, 4};
     const int cand_c[] = {2, 4, 8};
     t->cs = 1;
+    t->auto_shape = false;
     for (int th : cand_t) {
         for (int dp : cand_d) {
             if (!fused_lattice_valid_launch(h->g, th, dp)) continue;
@@ -1521,14 +1540,31 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
             best = ms_mode[i];
         }
     }
+    // the marching kernel, where it takes the lattice: no shape to choose
+    bool march = false;
+    t->auto_shape = true;
+    t->cs = 1;
+    t->staging = h->staging;
+    if (use_march(t)) {
+        const double ms = time_trajectories(t, reps, e0, e1);
+        if (ms > 0 && ms < best) {
+            best = ms;
+            march = true;
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     ising_hmc_destroy(t);
+    if (best_ms) *best_ms = best;
+    h->auto_shape = march;
+    if (march) {
+        h->cs = 1;
+        return ISING_OK;
+    }
     h->threads = bt;
     h->depth = bd;
     h->cs = bc;
     h->staging = stg;
-    if (best_ms) *best_ms = best;
     return ISING_OK;
 }
 
@@ -1542,7 +1578,7 @@ struct ising_group {
     std::vector<FusedArgs> args;
     std::vector<std::array<void *, 2>> argv;
     std::vector<cudaGraphNode_t> nodes;
-    std::vector<int> shape;  // threads, depth, CTAs per chain, bulk staging of every member
+    std::vector<int> shape;  // threads, depth, CTAs per chain, kernel_choice of every member
                              // at instantiation
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1599,7 +1635,7 @@ static ising_status group_build_graph(ising_group *g) {
         g->shape[4 * i] = h->threads;
         g->shape[4 * i + 1] = h->depth;
         g->shape[4 * i + 2] = h->cs;
-        g->shape[4 * i + 3] = staging_bulk(h);
+        g->shape[4 * i + 3] = kernel_choice(h);
     }
     cudaError_t e = cudaGraphInstantiate(&g->exec, g->graph, 0);
     if (e != cudaSuccess) return gfail(g, ISING_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
@@ -1656,7 +1692,7 @@ ising_status ising_group_trajectories_seeds(ising_group_t *g, int64_t n, const u
     // rebuild if a member's launch shape changed (autotune, set_launch)
     for (size_t i = 0; i < g->m.size(); ++i)
         if (g->shape[4 * i] != g->m[i]->threads || g->shape[4 * i + 1] != g->m[i]->depth ||
-            g->shape[4 * i + 2] != g->m[i]->cs || g->shape[4 * i + 3] != staging_bulk(g->m[i])) {
+            g->shape[4 * i + 2] != g->m[i]->cs || g->shape[4 * i + 3] != kernel_choice(g->m[i])) {
             ising_status st = group_build_graph(g);
             if (st != ISING_OK) return st;
             break;
@@ -1681,7 +1717,7 @@ ising_status ising_group_trajectories_seeds(ising_group_t *g, int64_t n, const u
             ising_hmc *h = g->m[i];
             g->args[i] = fused_args(h);
             g->args[i].mode = MODE_TRAJ;
-            g->args[i].seed = seeds[i];
+            set_seed(g->args[i], seeds[i]);
             g->args[i].traj0 = (uint32_t)(h->traj + done);
             g->args[i].n_traj = (int)k;
             g->args[i].eval_start = done == 0 && h->eval_pending;
