@@ -230,13 +230,15 @@ int64_t ising_hmc_launch_count(const ising_hmc_t *h);
 /* Synchronise the handle's stream; ETIMEOUT if a device wait gave up. */
 ising_status ising_hmc_sync(ising_hmc_t *h);
 
-/* 2D lattices (rows of at most 1024 sites, at least 24 rows) whose launch shape
- * and plane staging were left to the library and whose chains are not split run
- * on a kernel that marches down the rows and takes several force evaluations
- * per sweep; it has no shape to choose.  Its psi and p are bit for bit those of
- * the plane-streaming kernel below, which a call of ising_hmc_set_launch,
- * ising_hmc_set_chain_split or ising_hmc_set_staging selects; the FP64 sums
- * (action, energies, estimators) equal them to rounding.
+/* Lattices whose launch shape was left to the library run on
+ * kernels that march through the planes with register windows and have no shape
+ * to choose: in 2D (rows of at most 1024 sites, at least 24 rows, chains not
+ * split) with several force evaluations per sweep, in 3D (rows a multiple of 4)
+ * on as many CTAs per chain as ising_hmc_set_chain_split asked for or, if it
+ * was not called, the library picks for the number of chains.  Their psi and p
+ * are bit for bit those of the plane-streaming kernel below, which a call of
+ * ising_hmc_set_launch selects (as does, in 2D, a split); the FP64 sums (action, energies, estimators) equal them to rounding
+ * and depend on nothing but the handle.
  *
  * Launch shape of the fused FP32 lattice kernel: threads per CTA (a multiple
  * of 32, at most 4 float4 vectors of a plane per thread; 32..256 with one CTA
@@ -259,14 +261,13 @@ ising_status ising_hmc_get_launch(const ising_hmc_t *h, int *threads, int *depth
 ising_status ising_hmc_set_chain_split(ising_hmc_t *h, int ctas);
 int ising_hmc_get_chain_split(const ising_hmc_t *h);
 
-/* How the fused FP32 lattice kernel stages psi and p planes into its
- * shared-memory rings (Sec. 3's force evaluation streams the lattice plane by
+/* How the plane-streaming FP32 lattice kernel (see ising_hmc_set_launch) stages
+ * psi and p planes into its shared-memory rings (Sec. 3's force evaluation streams the lattice plane by
  * plane): ISING_STAGING_THREADS, every thread copies its share of a plane
  * with cp.async; ISING_STAGING_BULK, one lane issues each plane as a bulk
  * copy completing on an mbarrier (planes of whole 16-byte vectors: rows of a
  * multiple of 4 sites); ISING_STAGING_AUTO (default), bulk for planes of at
- * least 4 KB.  Results are bit for bit the same in both modes, and psi and p
- * under the automatic choice as well.  EINVAL for
+ * least 4 KB.  Results are bit for bit the same in every mode.  EINVAL for
  * other forms, unknown modes, or bulk on rows that are not a multiple of 4. */
 enum { ISING_STAGING_AUTO = 0, ISING_STAGING_THREADS = 1, ISING_STAGING_BULK = 2 };
 ising_status ising_hmc_set_staging(ising_hmc_t *h, int mode);

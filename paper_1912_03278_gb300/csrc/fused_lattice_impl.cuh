@@ -48,7 +48,7 @@ constexpr int MAX_CS = 8;                    // CTAs per chain (portable cluster
 constexpr int XCH_WORDS = 8;                 // per-CTA sums exchanged in a cluster
 constexpr int MAX_BARS = 16;                 // copy-group mbarriers (one per psi ring slot)
 // block reduction (32 warps x 8 doubles), broadcast words, two exchange
-// buffers, the copy-group mbarriers
+// buffers, the copy-group mbarriers (or other words kept for a trajectory)
 constexpr int RED_BYTES = 32 * 8 * 8 + 16 + 2 * XCH_WORDS * 8 + MAX_BARS * 8;
 
 // F(z) trails u by LAG planes: with LAG = 1 a plane's force reads only u

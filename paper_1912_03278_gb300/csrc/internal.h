@@ -68,7 +68,7 @@ struct FusedArgs {
     int eval_start;          // lattice kernel: evaluate S and the observables of the start
                              // configuration in the first trajectory's first pass
     int bulk;                // lattice kernel: stage planes by bulk copies (16-byte planes)
-    int march;               // threads per slab of the marching kernel (0: another kernel)
+    int march;               // threads per slab of a marching kernel (0: another kernel)
     int *err;
 };
 
@@ -118,6 +118,11 @@ int fused_lattice_valid_split(const Geometry &g, int threads, int depth, int cs)
 // kernel-node parameters.
 int march_lattice_threads(const Geometry &g);
 cudaError_t march_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args);
+// The same in 3D (rows a multiple of four long; one CTA or a cluster per chain).
+int march3_lattice_threads(const Geometry &g);
+cudaError_t march3_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args);
+// CTAs per chain for a launch of this many chains when none was asked for.
+int march3_lattice_split(const Geometry &g, int n_chains);
 // Cluster size of a graph kernel node made from fused_lattice_node (cs > 1).
 cudaError_t fused_lattice_node_cluster(cudaGraphNode_t node, int cs);
 int fused_lattice_pick(const Geometry &g, int *threads, int *depth);

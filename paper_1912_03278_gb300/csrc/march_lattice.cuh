@@ -186,12 +186,14 @@ struct Totals {
 };
 
 // Action terms of four sites (vector_action's formulas and values) in pair
-// arithmetic, the estimators and the conditional spin draws.
-template <bool RAG, bool HF, int NE>
+// arithmetic, the estimators and the conditional spin draws.  ym, yp: the rows
+// before and after in the plane (3D, else null).
+template <bool RAG, bool HF, int NE, bool D3 = false>
 __device__ __forceinline__ void row_action(const FusedArgs &A, const ChainParams &prm, const ActPairs &kc,
                                            const Row &c, const Row &zm, const Row &zp, float lw, float rx,
                                            const Row &t, const float (&hf)[4], int m, uint32_t site0,
-                                           const float (&su)[4], const float4 *tab, ActSums<NE> &ac) {
+                                           const float (&su)[4], const float4 *tab, ActSums<NE> &ac,
+                                           const Row *ym = nullptr, const Row *yp = nullptr) {
     float l[4], r[4];
     x_neighbours<RAG>(c, lw, rx, m, l, r);
     const bool has_h = HF || prm.hp != 0.0;
@@ -203,6 +205,10 @@ __device__ __forceinline__ void row_action(const FusedArgs &A, const ChainParams
     for (int q = 0; q < 2; ++q) {
         const pair_t ps = q ? c.b : c.a;
         f2x2 nb = two_sum(pk(l[2 * q], l[2 * q + 1]), pk(r[2 * q], r[2 * q + 1]));
+        if constexpr (D3) {
+            nb = df_add_f(nb, q ? ym->b : ym->a);
+            nb = df_add_f(nb, q ? yp->b : yp->a);
+        }
         nb = df_add_f(nb, q ? zm.b : zm.a);
         nb = df_add_f(nb, q ? zp.b : zp.a);
         const f2x2 a = df_add_q(df_mul_fc(kc.C, kc.neg_C, ps), df_mul(kc.bJ, kc.neg_bJ, nb));

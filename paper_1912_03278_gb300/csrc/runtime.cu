@@ -47,6 +47,7 @@ struct ising_hmc {
     // no launch shape asked for: the library may run trajectories on the
     // marching kernel, which has one shape per lattice
     bool auto_shape = true;
+    bool auto_split = true;   // no split asked for: the 3D marching kernel chooses one
     // FP32 lattice form: the configurations were set from outside and their
     // action is evaluated by the next trajectory's first force pass
     bool eval_pending = false;
@@ -377,15 +378,16 @@ static int staging_bulk(const ising_hmc *h) {
     return (int64_t)g.P * 4 >= BULK_AUTO_MIN_BYTES;
 }
 
-// Trajectories on the marching kernel: 2D chains on one CTA each, unless a
-// launch shape or a plane staging (choices of the plane-streaming kernel) was
-// asked for.  The kernel's threads per chain, 0 for the other kernels.
+// Trajectories on a marching kernel -- 2D chains on one CTA each, 3D chains on
+// one CTA or a cluster -- unless a launch shape (a choice of the plane-streaming
+// kernel) was asked for.  The kernel's threads, 0 for the plane-streaming kernel.
 static int use_march(const ising_hmc *h) {
-    const bool may = is_fp32_lattice(h) && h->auto_shape && h->cs == 1 && h->staging == ISING_STAGING_AUTO;
-    return may ? march_lattice_threads(h->g) : 0;
+    if (!is_fp32_lattice(h) || !h->auto_shape) return 0;
+    if (h->dim == 3) return march3_lattice_threads(h->g);
+    return h->cs == 1 ? march_lattice_threads(h->g) : 0;
 }
 // What of a handle, besides its shape and split, selects the kernel.
-static int kernel_choice(const ising_hmc *h) { return staging_bulk(h) | (use_march(h) ? 2 : 0); }
+static int kernel_choice(const ising_hmc *h) { return staging_bulk(h) | (use_march(h) ? 2 : 0) | (h->auto_split ? 4 : 0); }
 static FusedArgs fused_args(ising_hmc *h) {
     FusedArgs a{};
     for (int i = 0; i < 3; ++i) a.psi[i] = (float *)h->psi[i];
@@ -403,6 +405,16 @@ static FusedArgs fused_args(ising_hmc *h) {
     a.bulk = staging_bulk(h);
     a.march = use_march(h);
     a.err = h->d_err;
+    return a;
+}
+
+// Arguments of a launch of trajectories.  The split the library chooses depends
+// on the handle alone, so that a group's launch and the handle's own give the
+// same results bit for bit.
+static FusedArgs trajectory_args(ising_hmc *h) {
+    FusedArgs a = fused_args(h);
+    a.mode = MODE_TRAJ;
+    if (a.march && h->dim == 3 && h->auto_split) a.cs = march3_lattice_split(h->g, h->n_chains);
     return a;
 }
 
@@ -1013,8 +1025,7 @@ static ising_status run_trajectories(ising_hmc *h, int64_t n, uint64_t seed) {
         int64_t done = 0;
         while (done < n) {
             const int64_t k = std::min(per, n - done);
-            FusedArgs a = fused_args(h);
-            a.mode = MODE_TRAJ;
+            FusedArgs a = trajectory_args(h);
             set_seed(a, seed);
             a.traj0 = (uint32_t)(h->traj + done);
             a.n_traj = (int)k;
@@ -1370,6 +1381,7 @@ ising_status ising_hmc_set_chain_split(ising_hmc_t *h, int ctas) {
         return fail(h, ISING_EINVAL, "invalid chain split %d (threads=%d depth=%d, %d planes)", ctas,
                     h->threads, h->depth, h->g.nplanes);
     h->cs = ctas;
+    h->auto_split = false;
     return ISING_OK;
 }
 
@@ -1435,6 +1447,7 @@ static ising_status clone_for_tuning(ising_hmc *h, int nt, ising_hmc **out) {
         (*out)->cs = h->cs;
         (*out)->staging = h->staging;
         (*out)->auto_shape = h->auto_shape;
+        (*out)->auto_split = h->auto_split;
     }
     return st;
 }
@@ -1486,7 +1499,7 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
     const int cand_d[] = {1, 2, 4};
     const int cand_c[] = {2, 4, 8};
     t->cs = 1;
-    t->auto_shape = false;
+    t->auto_shape = t->auto_split = false;
     for (int th : cand_t) {
         for (int dp : cand_d) {
             if (!fused_lattice_valid_launch(h->g, th, dp)) continue;
@@ -1540,15 +1553,18 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
             best = ms_mode[i];
         }
     }
-    // the marching kernel, where it takes the lattice: no shape to choose
+    // the marching kernels, where they take the lattice: no shape to choose,
+    // in 3D a split
     bool march = false;
     t->auto_shape = true;
-    t->cs = 1;
     t->staging = h->staging;
-    if (use_march(t)) {
+    for (int c : {1, 2, 4, 8}) {
+        t->cs = c;
+        if (!use_march(t) || (c > 1 && h->g.nplanes < 2 * c)) continue;
         const double ms = time_trajectories(t, reps, e0, e1);
         if (ms > 0 && ms < best) {
             best = ms;
+            bc = c;
             march = true;
         }
     }
@@ -1557,8 +1573,9 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
     ising_hmc_destroy(t);
     if (best_ms) *best_ms = best;
     h->auto_shape = march;
+    h->auto_split = false;
     if (march) {
-        h->cs = 1;
+        h->cs = bc;
         return ISING_OK;
     }
     h->threads = bt;
@@ -1623,14 +1640,13 @@ static ising_status group_build_graph(ising_group *g) {
     });
     for (size_t i : order) {
         ising_hmc *h = g->m[i];
-        g->args[i] = fused_args(h);
-        g->args[i].mode = MODE_TRAJ;
+        g->args[i] = trajectory_args(h);
         g->args[i].n_traj = 1;
         g->argv[i] = {&g->args[i], &h->sched};
         cudaKernelNodeParams np;
         cudaError_t e = fused_lattice_node(g->args[i], h->threads, h->depth, &np, g->argv[i].data());
         if (e == cudaSuccess) e = cudaGraphAddKernelNode(&g->nodes[i], g->graph, nullptr, 0, &np);
-        if (e == cudaSuccess && h->cs > 1) e = fused_lattice_node_cluster(g->nodes[i], h->cs);
+        if (e == cudaSuccess && g->args[i].cs > 1) e = fused_lattice_node_cluster(g->nodes[i], g->args[i].cs);
         if (e != cudaSuccess) return gfail(g, ISING_ECUDA, "graph node: %s", cudaGetErrorString(e));
         g->shape[4 * i] = h->threads;
         g->shape[4 * i + 1] = h->depth;
@@ -1715,8 +1731,7 @@ ising_status ising_group_trajectories_seeds(ising_group_t *g, int64_t n, const u
         const int64_t k = std::min(per, n - done);
         for (size_t i = 0; i < g->m.size(); ++i) {
             ising_hmc *h = g->m[i];
-            g->args[i] = fused_args(h);
-            g->args[i].mode = MODE_TRAJ;
+            g->args[i] = trajectory_args(h);
             set_seed(g->args[i], seeds[i]);
             g->args[i].traj0 = (uint32_t)(h->traj + done);
             g->args[i].n_traj = (int)k;
@@ -1821,33 +1836,50 @@ ising_status ising_group_autotune(ising_group_t *g, int reps, double *best_ms) {
             unsplit_ok &= fused_lattice_valid_split(tmp[i]->g, tmp[i]->threads, tmp[i]->depth, 1) != 0;
         }
         if (any && unsplit_ok) {
-            for (size_t i = 0; i < n; ++i) tmp[i]->cs = 1;
+            std::vector<bool> was(n);
+            for (size_t i = 0; i < n; ++i) {
+                was[i] = tmp[i]->auto_split;
+                tmp[i]->cs = 1;
+                tmp[i]->auto_split = false;
+            }
             const double t1 = time_group();
             if (t1 > 0 && (best < 0 || t1 < best)) best = t1;
             else
-                for (size_t i = 0; i < n; ++i) tmp[i]->cs = cur[i];
+                for (size_t i = 0; i < n; ++i) {
+                    tmp[i]->cs = cur[i];
+                    tmp[i]->auto_split = was[i];
+                }
         }
     }
     for (int round = 0; round < 2; ++round) {
         for (size_t i : order) {
             ising_hmc *t = tmp[i];
             const int keep = t->cs;
+            const bool keep_auto = t->auto_split;
             int bc = keep;
+            bool ba = keep_auto;
             for (int c : {1, 2, 4, 8}) {
-                if (c == keep || !fused_lattice_valid_split(t->g, t->threads, t->depth, c)) continue;
+                if ((c == keep && !keep_auto) || !fused_lattice_valid_split(t->g, t->threads, t->depth, c))
+                    continue;
                 t->cs = c;
+                t->auto_split = false;
                 const double ms = time_group();
                 if (ms > 0 && (best < 0 || ms < best)) {
                     best = ms;
                     bc = c;
+                    ba = false;
                 }
             }
             t->cs = bc;
+            t->auto_split = ba;
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    for (size_t i = 0; i < n; ++i) g->m[i]->cs = tmp[i]->cs;
+    for (size_t i = 0; i < n; ++i) {
+        g->m[i]->cs = tmp[i]->cs;
+        g->m[i]->auto_split = tmp[i]->auto_split;
+    }
     cleanup();
     if (best_ms) *best_ms = best;
     return best > 0 ? ISING_OK : gfail(g, ISING_ECUDA, "group autotune: no launch succeeded");
