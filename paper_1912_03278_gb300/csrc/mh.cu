@@ -38,6 +38,7 @@ namespace {
 constexpr uint32_t PURPOSE_MH = 5;
 constexpr int MH_THREADS = 256;
 constexpr int MH_TAB = 13;   // neighbour sums -6..6
+constexpr int64_t MH_CLUSTER_WORDS = 4096;   // words per SM up to which sweeps run on clusters
 
 // Per-chain parameters and sums.
 struct MHChain {
@@ -51,12 +52,15 @@ struct MHArgs {
     const uint32_t *ttab;           // packed form, per chain: [2][8] thresholds, index (s > 0, count)
     const float *ptab;              // per chain: [2][MH_TAB], index (s > 0, nb + 6)
     unsigned long long *acc;        // per chain: M, B, flips (two's complement)
+    unsigned long long *acc_prev;   // packed form: the previous sweep's sums, still to be measured
     MHChain *chains;
     int X, Y, Z;
     int64_t N;
     uint64_t seed;
+    uint32_t rk[20];                // its Philox key schedule (packed form)
     uint32_t half;                  // 2 * sweep + colour
     int measure;
+    int measure_prev;               // -1: nothing pending
 };
 
 template <int DIM>
@@ -197,118 +201,12 @@ __global__ void __launch_bounds__(MH_THREADS) mh_colour_row8_kernel(MHArgs a, in
     }
 }
 
-// Multi-spin-coded form, rows a multiple of 32 long: 32 spins of a row per
-// 32-bit word (bit j = site x0 + j, set for spin +1).  A thread owns one word:
-// the neighbour words give the left/right neighbour bit-vectors by shifts
-// (the row's end bits from the adjacent words, periodic), the other
-// directions whole words; a bit-sliced adder counts each lane's +1
-// neighbours (cnt = (nb + 2 dim) / 2).  The 16 lanes of the launch's colour
-// take their decisions with the same Philox words as the byte kernels (site i
-// uses word (i/2) mod 4 of block i/8, so lane k0 + 2m uses word m & 3 of block
-// 4w + m/4) against an integer threshold: (x >> 9) < T with T the number of
-// 23-bit values k with (k + 1/2) 2^-23 < p, i.e. exactly the FP32 test
-// u23(x) < p.  Spins, flips and sums equal the byte kernels' bit for bit.
-__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
-    return (a & b) | (c & (a ^ b));
-}
-
-template <int DIM>
-__global__ void __launch_bounds__(MH_THREADS) mh_packed_kernel(MHArgs a, int colour) {
-    __shared__ uint32_t tt[16];
-    const int chain = blockIdx.y;
-    if (threadIdx.x < 16) tt[threadIdx.x] = a.ttab[chain * 16 + threadIdx.x];
-    __syncthreads();
-    const uint32_t X = (uint32_t)a.X, Y = (uint32_t)a.Y, Z = (uint32_t)a.Z;
-    const uint32_t XW = X >> 5;                        // words per row
-    const uint32_t nw = (uint32_t)(a.N >> 5);          // words per chain
-    const uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
-    int dM = 0, dB = 0, dF = 0;
-    if (w < nw) {
-        uint32_t *sw = a.sw + (int64_t)chain * nw;
-        const uint32_t row = w / XW;                   // 32-bit index arithmetic: N <= 2^31
-        const uint32_t xw = w - row * XW;
-        const uint32_t y = row % Y, z = row / Y;
-        const uint32_t c = sw[w];
-        const uint32_t wl = xw > 0 ? w - 1 : w + XW - 1;
-        const uint32_t wr = xw + 1 < XW ? w + 1 : w + 1 - XW;
-        const uint32_t Lv = (c << 1) | (sw[wl] >> 31);      // lane j: site x - 1
-        const uint32_t Rv = (c >> 1) | (sw[wr] << 31);      // lane j: site x + 1
-        uint32_t b0, b1, b2 = 0u;
-        if constexpr (DIM == 1) {
-            b0 = Lv ^ Rv;
-            b1 = Lv & Rv;
-        } else {
-            const uint32_t RW = XW * Y;                // words per plane
-            const uint32_t Uv = sw[y > 0 ? w - XW : w + (Y - 1) * XW];
-            const uint32_t Dv = sw[y + 1 < Y ? w + XW : w - (Y - 1) * XW];
-            if constexpr (DIM == 2) {
-                const uint32_t s1 = Lv ^ Rv, c1 = Lv & Rv, s2 = Uv ^ Dv, c2 = Uv & Dv;
-                b0 = s1 ^ s2;
-                const uint32_t k = s1 & s2;
-                b1 = c1 ^ c2 ^ k;
-                b2 = maj3(c1, c2, k);
-            } else {
-                const uint32_t Fv = sw[z > 0 ? w - RW : w + (Z - 1) * RW];
-                const uint32_t Bv = sw[z + 1 < Z ? w + RW : w - (Z - 1) * RW];
-                const uint32_t s1 = Lv ^ Rv ^ Uv, c1 = maj3(Lv, Rv, Uv);
-                const uint32_t s2 = Dv ^ Fv ^ Bv, c2 = maj3(Dv, Fv, Bv);
-                b0 = s1 ^ s2;
-                const uint32_t k = s1 & s2;
-                b1 = c1 ^ c2 ^ k;
-                b2 = maj3(c1, c2, k);
-            }
-        }
-        // lanes of this colour: j = k0 + 2m (x0 is a multiple of 32, so even)
-        const uint32_t k0 = (uint32_t)(colour + y + z) & 1u;
-        const uint32_t e0 = b0 >> k0, e1 = b1 >> k0, e2 = b2 >> k0, es = c >> k0;
-        uint32_t fl = 0u;   // flips, lane m at bit 2m
-#pragma unroll
-        for (int blk = 0; blk < 4; ++blk) {
-            const u32x4 r = philox(4 * w + (uint32_t)blk, a.half, (uint32_t)chain, PURPOSE_MH,
-                                   a.seed);
-            const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int m = 4 * blk + q, sh = 2 * m;
-                const uint32_t idx = ((es >> sh) & 1u) << 3 | ((e2 >> sh) & 1u) << 2 |
-                                     ((e1 >> sh) & 1u) << 1 | ((e0 >> sh) & 1u);
-                fl |= (uint32_t)((rw[q] >> 9) < tt[idx]) << sh;
-            }
-        }
-        const uint32_t lanes = 0x55555555u << k0;
-        const uint32_t flips = fl << k0;
-        const uint32_t nc = c ^ flips;
-        sw[w] = nc;
-        const int up = __popc(nc & lanes);
-        dM = 2 * up - 16;
-        dF = __popc(flips);
-        if (colour == 1) {
-            // sum over the lanes of s * nb, nb = 2 cnt - 2 DIM
-            const uint32_t pl = nc & lanes, mi = ~nc & lanes;
-            const int cp = __popc(b0 & pl) + 2 * __popc(b1 & pl) + 4 * __popc(b2 & pl);
-            const int cm = __popc(b0 & mi) + 2 * __popc(b1 & mi) + 4 * __popc(b2 & mi);
-            dB = (2 * cp - 2 * DIM * up) - (2 * cm - 2 * DIM * (16 - up));
-        }
-    }
-    dM = __reduce_add_sync(0xffffffffu, dM);
-    dB = __reduce_add_sync(0xffffffffu, dB);
-    dF = __reduce_add_sync(0xffffffffu, dF);
-    if ((threadIdx.x & 31) == 0) {
-        unsigned long long *acc = a.acc + 3 * chain;
-        if (dM) atomicAdd(acc + 0, (unsigned long long)(long long)dM);
-        if (dB) atomicAdd(acc + 1, (unsigned long long)(long long)dB);
-        if (dF) atomicAdd(acc + 2, (unsigned long long)(long long)dF);
-    }
-}
-
-// Observables of the sweep just finished (if measured), then clear the sums.
-__global__ void mh_measure_kernel(MHArgs a, int n_chains) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_chains) return;
-    unsigned long long *acc = a.acc + 3 * c;
-    const long long M = (long long)acc[0], B = (long long)acc[1], F = (long long)acc[2];
+// Observables of a finished sweep (if measured) from chain c's sums, which are
+// cleared.
+__device__ __forceinline__ void mh_measure(const MHArgs &a, unsigned long long *acc, int c, bool measure) {
+    const long long M = (long long)__ldcg(acc), B = (long long)__ldcg(acc + 1), F = (long long)__ldcg(acc + 2);
     acc[0] = acc[1] = acc[2] = 0ull;
-    if (!a.measure) return;
+    if (!measure) return;
     // explicitly rounded operations in the order written (no contraction),
     // so the sums are reproducible bit for bit
     MHChain &ch = a.chains[c];
@@ -328,6 +226,186 @@ __global__ void mh_measure_kernel(MHArgs a, int n_chains) {
     sm[ISING_SUM_ABSM2] = __dadd_rn(sm[ISING_SUM_ABSM2], m2);
 }
 
+__global__ void mh_measure_kernel(MHArgs a, int n_chains) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < n_chains) mh_measure(a, a.acc + 3 * c, c, a.measure != 0);
+}
+
+// Multi-spin-coded form, rows a multiple of 32 long: 32 spins of a row per
+// 32-bit word (bit j = site x0 + j, set for spin +1).  A thread owns one word:
+// the neighbour words give the left/right neighbour bit-vectors by shifts
+// (the row's end bits from the adjacent words, periodic), the other
+// directions whole words; a bit-sliced adder counts each lane's +1
+// neighbours (cnt = (nb + 2 dim) / 2).  The 16 lanes of the launch's colour
+// take their decisions with the same Philox words as the byte kernels (site i
+// uses word (i/2) mod 4 of block i/8, so lane k0 + 2m uses word m & 3 of block
+// 4w + m/4) against an integer threshold: (x >> 9) < T with T the number of
+// 23-bit values k with (k + 1/2) 2^-23 < p, i.e. exactly the FP32 test
+// u23(x) < p.  Spins, flips and sums equal the byte kernels' bit for bit.
+__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
+    return (a & b) | (c & (a ^ b));
+}
+
+// 32 spins per word to one byte (+1 or -1) per spin.
+__global__ void __launch_bounds__(MH_THREADS) mh_unpack_kernel(const uint32_t *__restrict__ w,
+                                                               uint4 *__restrict__ out, int64_t nw) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // half a word per thread
+    if (i >= 2 * nw) return;
+    const uint32_t v = w[i >> 1] >> (16 * (i & 1));
+    uint32_t b[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        // four bits to the low bits of four bytes; 1 -> 0x01, 0 -> 0xff
+        const uint32_t n = (v >> (4 * k)) & 15u;
+        const uint32_t s = (n | (n << 7) | (n << 14) | (n << 21)) & 0x01010101u;
+        b[k] = s | ((s ^ 0x01010101u) * 0xffu);
+    }
+    out[i] = make_uint4(b[0], b[1], b[2], b[3]);
+}
+
+// One word's decisions of one colour; adds its spin sum, bond sum and flips.
+// L2: neighbouring words are read past L1 (another CTA may have written them).
+template <int DIM, bool L2>
+__device__ __forceinline__ void packed_word(const MHArgs &a, uint32_t *sw, const uint32_t *tt, uint32_t w,
+                                            int chain, int colour, uint32_t half, int &dM, int &dB,
+                                            int &dF) {
+    auto load = [&](uint32_t i) { return L2 ? __ldcg(sw + i) : sw[i]; };
+    const uint32_t X = (uint32_t)a.X, Y = (uint32_t)a.Y, Z = (uint32_t)a.Z;
+    const uint32_t XW = X >> 5;                        // words per row
+    const uint32_t row = w / XW;                       // 32-bit index arithmetic: N <= 2^31
+    const uint32_t xw = w - row * XW;
+    const uint32_t y = row % Y, z = row / Y;
+    const uint32_t c = load(w);
+    const uint32_t wl = xw > 0 ? w - 1 : w + XW - 1;
+    const uint32_t wr = xw + 1 < XW ? w + 1 : w + 1 - XW;
+    const uint32_t Lv = (c << 1) | (load(wl) >> 31);      // lane j: site x - 1
+    const uint32_t Rv = (c >> 1) | (load(wr) << 31);      // lane j: site x + 1
+    uint32_t b0, b1, b2 = 0u;
+    if constexpr (DIM == 1) {
+        b0 = Lv ^ Rv;
+        b1 = Lv & Rv;
+    } else {
+        const uint32_t RW = XW * Y;                // words per plane
+        const uint32_t Uv = load(y > 0 ? w - XW : w + (Y - 1) * XW);
+        const uint32_t Dv = load(y + 1 < Y ? w + XW : w - (Y - 1) * XW);
+        if constexpr (DIM == 2) {
+            const uint32_t s1 = Lv ^ Rv, c1 = Lv & Rv, s2 = Uv ^ Dv, c2 = Uv & Dv;
+            b0 = s1 ^ s2;
+            const uint32_t k = s1 & s2;
+            b1 = c1 ^ c2 ^ k;
+            b2 = maj3(c1, c2, k);
+        } else {
+            const uint32_t Fv = load(z > 0 ? w - RW : w + (Z - 1) * RW);
+            const uint32_t Bv = load(z + 1 < Z ? w + RW : w - (Z - 1) * RW);
+            const uint32_t s1 = Lv ^ Rv ^ Uv, c1 = maj3(Lv, Rv, Uv);
+            const uint32_t s2 = Dv ^ Fv ^ Bv, c2 = maj3(Dv, Fv, Bv);
+            b0 = s1 ^ s2;
+            const uint32_t k = s1 & s2;
+            b1 = c1 ^ c2 ^ k;
+            b2 = maj3(c1, c2, k);
+        }
+    }
+    // lanes of this colour: j = k0 + 2m (x0 is a multiple of 32, so even)
+    const uint32_t k0 = (uint32_t)(colour + y + z) & 1u;
+    // their table indices, four bits each (count, then spin), eight to a
+    // word: lanes of even m in ia, of odd m in ib
+    const uint32_t e01 = ((b0 >> k0) & 0x55555555u) | (((b1 >> k0) & 0x55555555u) << 1);
+    const uint32_t e2s = ((b2 >> k0) & 0x55555555u) | (((c >> k0) & 0x55555555u) << 1);
+    const uint32_t ia = (e01 & 0x33333333u) | ((e2s & 0x33333333u) << 2);
+    const uint32_t ib = ((e01 >> 2) & 0x33333333u) | (e2s & 0xccccccccu);
+    uint32_t fl = 0u;   // flips, lane m at bit 2m
+#pragma unroll
+    for (int blk = 0; blk < 4; ++blk) {
+        const u32x4 r = philox(4 * w + (uint32_t)blk, half, (uint32_t)chain, PURPOSE_MH, a.rk);
+        const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int m = 4 * blk + q;
+            const uint32_t idx = ((m & 1 ? ib : ia) >> (4 * (m >> 1))) & 15u;
+            if ((rw[q] >> 9) < tt[idx]) fl |= 1u << (2 * m);
+        }
+    }
+    const uint32_t lanes = 0x55555555u << k0;
+    const uint32_t flips = fl << k0;
+    const uint32_t nc = c ^ flips;
+    sw[w] = nc;
+    const int up = __popc(nc & lanes);
+    dM += 2 * up - 16;
+    dF += __popc(flips);
+    if (colour == 1) {
+        // sum over the lanes of s * nb, nb = 2 cnt - 2 DIM
+        const uint32_t pl = nc & lanes, mi = ~nc & lanes;
+        const int cp = __popc(b0 & pl) + 2 * __popc(b1 & pl) + 4 * __popc(b2 & pl);
+        const int cm = __popc(b0 & mi) + 2 * __popc(b1 & mi) + 4 * __popc(b2 & mi);
+        dB += (2 * cp - 2 * DIM * up) - (2 * cm - 2 * DIM * (16 - up));
+    }
+}
+
+__device__ __forceinline__ void add_sums(unsigned long long *acc, int dM, int dB, int dF) {
+    dM = __reduce_add_sync(0xffffffffu, dM);
+    dB = __reduce_add_sync(0xffffffffu, dB);
+    dF = __reduce_add_sync(0xffffffffu, dF);
+    if ((threadIdx.x & 31) == 0) {
+        if (dM) atomicAdd(acc + 0, (unsigned long long)(long long)dM);
+        if (dB) atomicAdd(acc + 1, (unsigned long long)(long long)dB);
+        if (dF) atomicAdd(acc + 2, (unsigned long long)(long long)dF);
+    }
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(MH_THREADS) mh_packed_kernel(const __grid_constant__ MHArgs a, int colour) {
+    __shared__ uint32_t tt[16];
+    const int chain = blockIdx.y;
+    if (threadIdx.x < 16) tt[threadIdx.x] = a.ttab[chain * 16 + threadIdx.x];
+    // the previous sweep's measurement, left to this launch (which adds to the
+    // other set of sums)
+    if (colour == 0 && blockIdx.x == 0 && threadIdx.x == 0 && a.measure_prev >= 0)
+        mh_measure(a, a.acc_prev + 3 * chain, chain, a.measure_prev != 0);
+    __syncthreads();
+    const uint32_t nw = (uint32_t)(a.N >> 5);          // words per chain
+    const uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
+    int dM = 0, dB = 0, dF = 0;
+    if (w < nw)
+        packed_word<DIM, false>(a, a.sw + (int64_t)chain * nw, tt, w, chain, colour, a.half, dM, dB, dF);
+    add_sums(a.acc + 3 * chain, dM, dB, dF);
+}
+
+// Whole sweeps of a chain on one cluster of CTAs, n sweeps per launch: where a
+// colour's launch is too short to fill the GPU, the launches' starts and ends
+// took most of the time (64 chains of L = 256: 16.3 us a sweep in two launches,
+// 7 us of them at the kernel's full rate).  Spins stay in global memory (in L2);
+// the CTAs meet at a cluster barrier after each colour.  The sums alternate
+// between two sets: rank 0 measures sweep k while sweep k + 1 adds to the other.
+template <int DIM>
+__global__ void __launch_bounds__(1024) mh_cluster_kernel(const __grid_constant__ MHArgs a, uint32_t sweep0,
+                                                          int n, int64_t n_therm, int n_chains) {
+    __shared__ uint32_t tt[16];
+    uint32_t cs, cr;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(cs));
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(cr));
+    const int chain = (int)(blockIdx.x / cs);
+    if (threadIdx.x < 16) tt[threadIdx.x] = a.ttab[chain * 16 + threadIdx.x];
+    __syncthreads();
+    const uint32_t nw = (uint32_t)(a.N >> 5);
+    uint32_t *sw = a.sw + (int64_t)chain * nw;
+    for (int k = 0; k < n; ++k) {
+        unsigned long long *acc = a.acc + 3 * ((int64_t)n_chains * (k & 1) + chain);
+        int dM = 0, dB = 0, dF = 0;
+#pragma unroll 1
+        for (int colour = 0; colour < 2; ++colour) {
+            for (uint32_t w = cr * blockDim.x + threadIdx.x; w < nw; w += cs * blockDim.x)
+                packed_word<DIM, true>(a, sw, tt, w, chain, colour, 2 * (sweep0 + (uint32_t)k) + (uint32_t)colour,
+                                       dM, dB, dF);
+            __syncwarp();
+            if (colour) add_sums(acc, dM, dB, dF);
+            asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+                         "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        }
+        if (cr == 0 && threadIdx.x == 0)
+            mh_measure(a, acc, chain, (int64_t)sweep0 + k >= n_therm);
+    }
+}
+
 thread_local char g_mh_create_err[512];
 
 }  // namespace
@@ -339,6 +417,7 @@ struct ising_mh {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     bool packed = false;            // rows a multiple of 32: 32 spins per word
+    int cluster = 0;                // packed: CTAs per chain of whole sweeps (0: a launch per colour)
     int8_t *s = nullptr;            // byte form: one int8 per spin
     uint32_t *sw = nullptr;         // packed form
     uint32_t *ttab = nullptr;       // packed form: per chain [2][8] thresholds
@@ -470,11 +549,31 @@ ising_status ising_mh_create(const ising_hmc_config *cfg, ising_mh_t **out) {
             return bail(mh_fail(h, ISING_ECUDA, "stream creation failed"));
         h->own_stream = true;
     }
+    // Whole sweeps on a cluster per chain (up to eight CTAs, as many as two of
+    // 1024 threads per SM allow): where the words of all chains are few, so that a
+    // colour's launch ends before it is under way, or where the clusters fill
+    // the GPU.  Per sweep, clusters / a launch per colour: 64 chains of L = 256 8.6 /
+    // 16.7 us, 300 of L = 64 5.6 / 12.3, 304 of L = 512 86 / 104; 100 of L = 512
+    // (a third of the GPU left out) 46 / 43.
+    if (h->packed) {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
+            const int64_t slots = 2 * (int64_t)sms;
+            int cs = 1;
+            while (cs < 8 && 2 * (int64_t)cs * C <= slots && N / 32 > 64 * cs) cs *= 2;
+            const int64_t ctas = (int64_t)cs * C, waves = (ctas + slots - 1) / slots;
+            if ((waves == 1 && (int64_t)C * (N / 32) <= MH_CLUSTER_WORDS * (int64_t)sms) ||
+                4 * ctas >= 3 * waves * slots)
+                h->cluster = cs;
+        }
+        cudaGetLastError();
+    }
     const size_t sb = h->packed ? (size_t)C * (N / 32) * 4 : (size_t)C * N;
     if ((h->packed ? cudaMalloc((void **)&h->sw, sb) : cudaMalloc((void **)&h->s, sb)) != cudaSuccess ||
         cudaMalloc((void **)&h->ttab, ttab.size() * sizeof(uint32_t)) != cudaSuccess ||
         cudaMalloc((void **)&h->ptab, tab.size() * sizeof(float)) != cudaSuccess ||
-        cudaMalloc((void **)&h->acc, (size_t)C * 3 * sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMalloc((void **)&h->acc, (size_t)C * 6 * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMalloc((void **)&h->chains, (size_t)C * sizeof(MHChain)) != cudaSuccess) {
         cudaGetLastError();
         return bail(mh_fail(h, ISING_ENOMEM, "device allocation failed (%zu bytes of spins)", sb));
@@ -484,7 +583,7 @@ ising_status ising_mh_create(const ising_hmc_config *cfg, ising_mh_t **out) {
                         h->stream) != cudaSuccess ||
         cudaMemcpyAsync(h->ttab, ttab.data(), ttab.size() * sizeof(uint32_t),
                         cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
-        cudaMemsetAsync(h->acc, 0, (size_t)C * 3 * sizeof(unsigned long long), h->stream) != cudaSuccess ||
+        cudaMemsetAsync(h->acc, 0, (size_t)C * 6 * sizeof(unsigned long long), h->stream) != cudaSuccess ||
         cudaMemcpyAsync(h->ptab, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice,
                         h->stream) != cudaSuccess ||
         cudaMemcpyAsync(h->chains, ch.data(), (size_t)C * sizeof(MHChain), cudaMemcpyHostToDevice,
@@ -516,15 +615,60 @@ ising_status ising_mh_sweeps(ising_mh_t *h, int64_t n, uint64_t seed) {
                              : mh_colour_row8_kernel<1>;
         grid.x = (unsigned)((groups + 2 * MH_THREADS - 1) / (2 * MH_THREADS));   // two groups per thread
     }
+    for (int r = 0; r < 10; ++r) {
+        a.rk[2 * r] = (uint32_t)seed + (uint32_t)r * 0x9E3779B9u;
+        a.rk[2 * r + 1] = (uint32_t)(seed >> 32) + (uint32_t)r * 0xBB67AE85u;
+    }
+    a.measure_prev = -1;
+    if (h->packed && h->cluster > 0) {
+        a.acc = h->acc;
+        // whole sweeps per launch, of bounded work
+        const int64_t per = std::max<int64_t>(1, std::min<int64_t>(4096, ((int64_t)1 << 34) / (h->N * h->n_chains)));
+        for (int64_t k = 0; k < n;) {
+            const int m = (int)std::min(per, n - k);
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)h->cluster;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.gridDim = dim3((unsigned)(h->n_chains * h->cluster));
+            const int64_t words = (h->N / 32 + h->cluster - 1) / h->cluster;
+            cfg.blockDim = dim3((unsigned)std::min<int64_t>(1024, (words + 31) / 32 * 32));
+            cfg.stream = h->stream;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            auto whole = h->dim == 3   ? mh_cluster_kernel<3>
+                         : h->dim == 2 ? mh_cluster_kernel<2>
+                                       : mh_cluster_kernel<1>;
+            const cudaError_t e = cudaLaunchKernelEx(&cfg, whole, a, (uint32_t)(h->sweep + k), m,
+                                                     (int64_t)h->n_therm, h->n_chains);
+            h->launches += 1;
+            if (e != cudaSuccess) return mh_fail(h, ISING_ECUDA, "sweep launch: %s", cudaGetErrorString(e));
+            k += m;
+        }
+        h->sweep += n;
+        return ISING_OK;
+    }
     for (int64_t k = 0; k < n; ++k) {
         const int64_t sw = h->sweep + k;
         a.measure = sw >= h->n_therm;
+        if (h->packed) {   // sums alternate between two sets, see below
+            a.acc_prev = h->acc + 3 * (size_t)h->n_chains * (size_t)((k + 1) & 1);
+            a.acc = h->acc + 3 * (size_t)h->n_chains * (size_t)(k & 1);
+        }
         for (int c = 0; c < 2; ++c) {
             a.half = (uint32_t)(2 * sw + c);
             kern<<<grid, MH_THREADS, 0, h->stream>>>(a, c);
         }
-        mh_measure_kernel<<<(h->n_chains + 127) / 128, 128, 0, h->stream>>>(a, h->n_chains);
-        h->launches += 3;
+        h->launches += 2;
+        // packed form: the next sweep's first launch measures this one; the
+        // last sweep of the call has a launch for it
+        if (h->packed && k + 1 < n) {
+            a.measure_prev = a.measure;
+        } else {
+            mh_measure_kernel<<<(h->n_chains + 127) / 128, 128, 0, h->stream>>>(a, h->n_chains);
+            h->launches += 1;
+        }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return mh_fail(h, ISING_ECUDA, "sweep launch: %s", cudaGetErrorString(e));
     }
@@ -566,12 +710,33 @@ ising_status ising_mh_get_spins(ising_mh_t *h, int8_t *out) {
     ising_status st = ising_mh_sync(h);
     if (st != ISING_OK) return st;
     if (h->packed) {
-        const size_t nw = (size_t)h->n_chains * (h->N / 32);
-        std::vector<uint32_t> w(nw);
-        if (cudaMemcpy(w.data(), h->sw, nw * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
-            return mh_fail(h, ISING_ECUDA, "%s", cudaGetErrorString(cudaGetLastError()));
-        for (size_t k = 0; k < nw; ++k)
-            for (int j = 0; j < 32; ++j) out[32 * k + j] = ((w[k] >> j) & 1u) ? 1 : -1;
+        // unpacked on the device, up to 64 MB at a time (the host's loop over
+        // the bits took about 1 ns per spin)
+        const int64_t nw = (int64_t)h->n_chains * (h->N / 32);
+        const int64_t step = std::min<int64_t>(nw, (int64_t)1 << 21);
+        void *buf = nullptr;
+        if (cudaMallocAsync(&buf, (size_t)step * 32, h->stream) != cudaSuccess) {
+            cudaGetLastError();   // no room: on the host
+            std::vector<uint32_t> w(nw);
+            if (cudaMemcpy(w.data(), h->sw, (size_t)nw * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
+                return mh_fail(h, ISING_ECUDA, "%s", cudaGetErrorString(cudaGetLastError()));
+            for (int64_t k = 0; k < nw; ++k)
+                for (int j = 0; j < 32; ++j) out[32 * k + j] = ((w[k] >> j) & 1u) ? 1 : -1;
+            return ISING_OK;
+        }
+        cudaError_t e = cudaSuccess;
+        for (int64_t k = 0; k < nw && e == cudaSuccess; k += step) {
+            const int64_t m = std::min(step, nw - k);
+            mh_unpack_kernel<<<(unsigned)((2 * m + MH_THREADS - 1) / MH_THREADS), MH_THREADS, 0, h->stream>>>(
+                h->sw + k, static_cast<uint4 *>(buf), m);
+            h->launches += 1;
+            e = cudaGetLastError();
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(out + 32 * k, buf, (size_t)m * 32, cudaMemcpyDeviceToHost, h->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        }
+        cudaFreeAsync(buf, h->stream);
+        if (e != cudaSuccess) return mh_fail(h, ISING_ECUDA, "%s", cudaGetErrorString(e));
         return ISING_OK;
     }
     if (cudaMemcpy(out, h->s, (size_t)h->n_chains * h->N, cudaMemcpyDeviceToHost) != cudaSuccess)
