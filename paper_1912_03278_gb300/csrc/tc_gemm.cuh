@@ -326,7 +326,10 @@ constexpr int SMEM_BYTES = (int)sizeof(Smem) + 1024;
 // TILE_M x TILE_N (K = nk * 128 bytes: 64 BF16 or, with FP8, 128 E4M3 elements per
 // stage row), each computed reps times: repetition r reads
 // A from row epi.a_off(r) on and B from row epi.b_off(r) on (stacked operand
-// planes) and hands r to the epilogue.  Single mode: CTA b takes tiles b, b +
+// planes) and hands r to the epilogue.  With groups > 1 a tile's repetitions are
+// divided among that many units of work (unit = group * tiles + tile), for
+// problems of fewer tiles than the GPU takes at once; the epilogues of a tile
+// then run on several CTAs.  Single mode: CTA b takes tiles b, b +
 // gridDim.x, ..., each with all its repetitions in order.  Pair mode:
 // clusters of two CTAs take tiles likewise; CTA r of a pair stages A rows
 // TILE_M*um + 128 r .. +127 and B rows TILE_N*un + 128 r .. +127, signalling
@@ -349,7 +352,7 @@ constexpr int SMEM_BYTES = (int)sizeof(Smem) + 1024;
 template <bool PAIR, class Epi, bool FP8 = false>
 __device__ __forceinline__ void gemm_persistent(const CUtensorMap *ta, const CUtensorMap *tb,
                                                 int m_units, int n_units, int nk, int reps,
-                                                Epi &epi, int *err) {
+                                                Epi &epi, int *err, int groups = 1) {
     using Md = Mode<PAIR>;
     constexpr int TN = Md::TILE_N;
     constexpr int KE = Elem<FP8>::BK_ELEMS;   // K elements per stage (128 bytes per row)
@@ -361,7 +364,9 @@ __device__ __forceinline__ void gemm_persistent(const CUtensorMap *ta, const CUt
     const bool leader = rank == 0;
     const int c0 = PAIR ? (int)cluster_id() : (int)blockIdx.x;
     const int nclu = PAIR ? (int)cluster_count() : (int)gridDim.x;
-    const int tiles = m_units * n_units;
+    const int tiles = m_units * n_units, units = tiles * groups;
+    // first repetition of unit u's group (of the next group: first_rep(u + tiles))
+    auto first_rep = [&](int u) { return u / tiles * reps / groups; };
     if (threadIdx.x == 0) {
         for (int i = 0; i < STAGES; ++i) {
             mbar_init(&s.full[i], 1);
@@ -388,10 +393,11 @@ __device__ __forceinline__ void gemm_persistent(const CUtensorMap *ta, const CUt
     if (warp == 0) {
         if (lane == 0) {
             uint32_t it = 0;
-            for (int u = c0; u < tiles && ok; u += nclu)
-            for (int r = 0; r < reps && ok; ++r) {
-                const int a_row = (u % m_units) * Md::TILE_M + (int)rank * BM + epi.a_off(r);
-                const int b_row = (u / m_units) * TN + (int)rank * BR + epi.b_off(r);
+            for (int u = c0; u < units && ok; u += nclu)
+            for (int r = first_rep(u); r < first_rep(u + tiles) && ok; ++r) {
+                const int t = u % tiles;
+                const int a_row = (t % m_units) * Md::TILE_M + (int)rank * BM + epi.a_off(r);
+                const int b_row = (t / m_units) * TN + (int)rank * BR + epi.b_off(r);
                 for (int kb = 0; kb < nk; ++kb, ++it) {
                     const uint32_t st = it % STAGES;
                     if (it >= STAGES) ok = mbar_wait(&s.empty[st], ((it / STAGES) & 1) ^ 1);
@@ -417,8 +423,8 @@ __device__ __forceinline__ void gemm_persistent(const CUtensorMap *ta, const CUt
         if (lane == 0 && leader) {
             constexpr uint32_t idesc = FP8 ? idesc_e4m3(Md::TILE_M, TN) : idesc_bf16(Md::TILE_M, TN);
             uint32_t it = 0, lt = 0;
-            for (int u = c0; u < tiles && ok; u += nclu)
-            for (int r = 0; r < reps && ok; ++r, ++lt) {
+            for (int u = c0; u < units && ok; u += nclu)
+            for (int r = first_rep(u); r < first_rep(u + tiles) && ok; ++r, ++lt) {
                 const uint32_t buf = lt & 1;
                 if (lt >= 2)
                     ok = PAIR ? mbar_wait_cluster(&s.acc_empty[buf], ((lt >> 1) & 1) ^ 1)
@@ -457,14 +463,14 @@ __device__ __forceinline__ void gemm_persistent(const CUtensorMap *ta, const CUt
         const int g = (warp - 2) >> 2;
         const uint32_t empty0 = PAIR ? peer_addr(smem_u32(&s.acc_empty[0]), 0) : 0;
         uint32_t lt = 0;
-        for (int u = c0; u < tiles && ok; u += nclu)
-        for (int r = 0; r < reps && ok; ++r, ++lt) {
+        for (int u = c0; u < units && ok; u += nclu)
+        for (int r = first_rep(u); r < first_rep(u + tiles) && ok; ++r, ++lt) {
             const uint32_t buf = lt & 1;
             ok = mbar_wait(&s.acc_full[buf], (lt >> 1) & 1);
             if (!ok) break;
             tc_fence_after();
-            const int m0 = (u % m_units) * Md::TILE_M + (int)rank * BM;
-            const int n0 = (u / m_units) * TN;
+            const int m0 = (u % tiles % m_units) * Md::TILE_M + (int)rank * BM;
+            const int n0 = (u % tiles / m_units) * TN;
             const int row = q * 32 + lane;
             const uint32_t base = tmem + buf * TN + ((uint32_t)(q * 32) << 16);
             constexpr int EW = Epi::W;
