@@ -23,11 +23,17 @@
 // proposal's action to FP64 accuracy in double-float arithmetic, the kinetic
 // energies and the Sec. 4 estimators; the CTA takes the Metropolis decision
 // itself (as the lattice kernel does).
+//
+// The updates and the action run on pairs of sites in packed FP32 instructions
+// (pair.cuh: the scalar operations' bits): the resident kernel is bound by issue
+// (2432 chains of N = 4096: 0.50 -> 0.47 ms per call of one trajectory), the streaming
+// one by issue and latency (304 chains of N = 50001: 1.35 -> 1.14 ms).
 #include <cuda_runtime.h>
 
 #include "df32.cuh"
 #include "device_common.cuh"
 #include "internal.h"
+#include "pair.cuh"
 
 namespace ihmc {
 namespace {
@@ -38,30 +44,49 @@ constexpr int INF_MAX_THREADS = 256;
 // zero and are never stored.  V4: N is a multiple of 4, so a quad is one
 // aligned float4.
 struct Quad {
-    float v[4];
+    pair_t a, b;   // held as pairs: the updates run on two sites per instruction
 };
+__device__ __forceinline__ Quad make_quad(float v0, float v1, float v2, float v3) {
+    return Quad{pk(v0, v1), pk(v2, v3)};
+}
+__device__ __forceinline__ Quad make_quad(const float4 &t) { return make_quad(t.x, t.y, t.z, t.w); }
+__device__ __forceinline__ void unpack(const Quad &q, float (&v)[4]) {
+    upk(q.a, v[0], v[1]);
+    upk(q.b, v[2], v[3]);
+}
+__device__ __forceinline__ float4 to_float4(const Quad &q) {
+    float v[4];
+    unpack(q, v);
+    return make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ Quad quad_neg(const Quad &q) {
+    const pair_t m = pk1(-1.0f);
+    return Quad{mul2(q.a, m), mul2(q.b, m)};
+}
 
 template <bool V4>
 __device__ __forceinline__ Quad ldq(const float *__restrict__ base, int64_t i0, int64_t N) {
-    Quad r;
     if constexpr (V4) {
-        const float4 t = *reinterpret_cast<const float4 *>(base + i0);
-        r.v[0] = t.x; r.v[1] = t.y; r.v[2] = t.z; r.v[3] = t.w;
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(base + i0);
+        return Quad{t.x, t.y};
     } else {
+        float v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) r.v[k] = (i0 + k < N) ? base[i0 + k] : 0.0f;
+        for (int k = 0; k < 4; ++k) v[k] = (i0 + k < N) ? base[i0 + k] : 0.0f;
+        return make_quad(v[0], v[1], v[2], v[3]);
     }
-    return r;
 }
 
 template <bool V4>
 __device__ __forceinline__ void stq(float *__restrict__ base, int64_t i0, int64_t N, const Quad &r) {
     if constexpr (V4) {
-        *reinterpret_cast<float4 *>(base + i0) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+        *reinterpret_cast<ulonglong2 *>(base + i0) = make_ulonglong2(r.a, r.b);
     } else {
+        float v[4];
+        unpack(r, v);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (i0 + k < N) base[i0 + k] = r.v[k];
+            if (i0 + k < N) base[i0 + k] = v[k];
     }
 }
 
@@ -95,6 +120,7 @@ struct InfConst {
     f2 C2, k2, hp2, beta2;
     float Cf, kf, betaf, hpf;
     bool hzero;
+    const uint32_t *rk, *rk0;   // Philox key schedules of the seed and of key 0
 };
 
 __device__ __forceinline__ InfConst inf_const(const ChainParams &prm) {
@@ -115,18 +141,23 @@ __device__ __forceinline__ float field_f(const FusedArgs &A, const InfConst &kc,
     return A.hdf ? kc.betaf * A.hdf[i].x : kc.hpf;
 }
 
+// h' of the quad's sites.
+__device__ __forceinline__ Quad quad_field(const FusedArgs &A, const InfConst &kc, int64_t i0, int n) {
+    if (!A.hdf) return Quad{pk1(kc.hpf), pk1(kc.hpf)};
+    float h[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) h[k] = (k < n) ? field_f(A, kc, i0 + k) : 0.0f;
+    return make_quad(h[0], h[1], h[2], h[3]);
+}
+
 // t_i = tanh((A x)_i + h'_i) for the quad, with Sf = sum_j x_j in FP32: the
 // one formula both the force sweeps and the estimators use.
 __device__ __forceinline__ Quad quad_tanh(const FusedArgs &A, const InfConst &kc, const Quad &x,
                                           float Sf, int64_t i0, int n) {
-    Quad t;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float hf = (k < n) ? field_f(A, kc, i0 + k) : 0.0f;
-        const float a = fmaf(kc.Cf, x.v[k], kc.kf * (Sf - x.v[k]));
-        t.v[k] = tanh_f(a + hf);
-    }
-    return t;
+    const Quad h = quad_field(A, kc, i0, n);
+    const pair_t C = pk1(kc.Cf), k = pk1(kc.kf), S = pk1(Sf);
+    return Quad{tanh2(add2(fma2(C, x.a, mul2(k, sub2(S, x.a))), h.a)),
+                tanh2(add2(fma2(C, x.b, mul2(k, sub2(S, x.b))), h.b))};
 }
 
 // Action terms of the quad's sites of S(x) (Sec. 2, Eq. phi_psi_substitution:
@@ -136,34 +167,50 @@ __device__ __forceinline__ Quad quad_tanh(const FusedArgs &A, const InfConst &kc
 // draw per site.
 __device__ __forceinline__ void quad_action(const FusedArgs &A, const InfConst &kc, const Quad &x,
                                             const Quad &t, f2 Sx, int64_t i0, int n,
-                                            uint32_t spin_traj, uint64_t seed, int chain,
+                                            uint32_t spin_traj, const uint32_t *seed, int chain,
                                             const float4 *tab, Acc &acc) {
-    const float4 w = spin_u4_f32((uint32_t)(i0 >> 2), spin_traj, (uint32_t)chain, seed);
+    const float4 w = spin_u4((uint32_t)(i0 >> 2), spin_traj, (uint32_t)chain, seed);
     const float su[4] = {w.x, w.y, w.z, w.w};
     const bool has_h = A.hdf || !kc.hzero;
+    f2 si[4];
+    float ahi[4], tv[4], hf[4];
+    unpack(t, tv);
+    unpack(quad_field(A, kc, i0, n), hf);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {   // sites beyond n are computed and left out below
+        const pair_t ps = q ? x.b : x.a;
+        // sum over j != i
+        const f2x2 off = df_add_f(f2x2{pk1(Sx.hi), pk1(Sx.lo)}, mul2(ps, pk1(-1.0f)));
+        const f2x2 C2 = dup_df(kc.C2), k2 = dup_df(kc.k2);
+        const f2x2 a = df_add_q(df_mul_fc(C2, pk1(-kc.C2.hi), ps), df_mul(k2, pk1(-kc.k2.hi), off));
+        f2x2 y = a;
+        if (A.hdf) {
+            f2 h0{0.0f, 0.0f}, h1{0.0f, 0.0f};
+            if (2 * q < n) {
+                const float2 hh = A.hdf[i0 + 2 * q];
+                h0 = df_mul(kc.beta2, f2{hh.x, hh.y});
+            }
+            if (2 * q + 1 < n) {
+                const float2 hh = A.hdf[i0 + 2 * q + 1];
+                h1 = df_mul(kc.beta2, f2{hh.x, hh.y});
+            }
+            y = df_add_q(a, f2x2{pk(h0.hi, h1.hi), pk(h0.lo, h1.lo)});
+        } else if (!kc.hzero) {
+            y = df_add_q(a, dup_df(kc.hp2));
+        }
+        upk(action_term(ps, a, y, tab), si[2 * q], si[2 * q + 1]);
+        upk(a.hi, ahi[2 * q], ahi[2 * q + 1]);
+    }
     f2 sv{0.0f, 0.0f};
     float vT = 0.0f, vAT = 0.0f, vHT = 0.0f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if (k >= n) break;
-        const float ps = x.v[k];
-        const f2 off = df_add_f(Sx, -ps);   // sum over j != i
-        const f2 a = df_add_q(df_mul_f(kc.C2, ps), df_mul(kc.k2, off));
-        f2 y = a;
-        if (A.hdf) {
-            const float2 hh = A.hdf[i0 + k];
-            y = df_add_q(a, df_mul(kc.beta2, f2{hh.x, hh.y}));
-        } else if (!kc.hzero) {
-            y = df_add_q(a, kc.hp2);
-        }
-        const f2 ay = y.hi < 0.0f ? df_neg(y) : y;
-        const f2 gl = log1pexp_neg(f2{2.0f * ay.hi, 2.0f * ay.lo}, tab);
-        sv = df_add_q(sv, df_add_q(df_mul_f(a, 0.5f * ps), df_neg(df_add_q(ay, gl))));
-        const float tq = t.v[k];
-        vT += tq;
-        vAT = fmaf(a.hi, tq, vAT);
-        if (has_h) vHT = fmaf(field_f(A, kc, i0 + k), tq, vHT);
-        acc.sS += (su[k] < (1.0f + tq) * 0.5f) ? 1 : -1;
+        sv = k ? df_add_q(sv, si[k]) : si[k];
+        vT += tv[k];
+        vAT = fmaf(ahi[k], tv[k], vAT);
+        if (has_h) vHT = fmaf(hf[k], tv[k], vHT);
+        acc.sS += (su[k] < (1.0f + tv[k]) * 0.5f) ? 1 : -1;
     }
     acc_add(acc.S, acc.Slo, sv);
     kahan_add(acc.sT, acc.cT, vT);
@@ -179,11 +226,35 @@ __device__ __forceinline__ float *sel3(const FusedArgs &A, int i) {
 // quad sums in the same order (thread t: quads t, t + nt, ...; then the block
 // sum), so the sum kept while drifting equals the one recomputed from the
 // stored buffer bit for bit, and the force stays a function of psi alone.
-__device__ __forceinline__ float quad_sum(const Quad &v, int n) {
-    const float a = v.v[0] + (n > 1 ? v.v[1] : 0.0f);
-    const float b = (n > 2 ? v.v[2] : 0.0f) + (n > 3 ? v.v[3] : 0.0f);
+__device__ __forceinline__ float quad_sum(const Quad &q, int n) {
+    float v[4];
+    unpack(q, v);
+    const float a = v[0] + (n > 1 ? v[1] : 0.0f);
+    const float b = (n > 2 ? v[2] : 0.0f) + (n > 3 ? v[3] : 0.0f);
     return a + b;
 }
+
+// Kinetic energy of the quad's first n sites, added site by site.
+__device__ __forceinline__ void quad_kinetic(const Quad &p, int n, f2 &K, float &Klo) {
+    f2 v[4];
+    upk(half_square(p.a), v[0], v[1]);
+    upk(half_square(p.b), v[2], v[3]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (k < n) acc_add(K, Klo, v[k]);
+}
+
+// p += kick F with F = A u, and x + drift p.
+__device__ __forceinline__ Quad quad_kick(const InfConst &kc, float kick, const Quad &p, const Quad &u, float Uf) {
+    const pair_t C = pk1(kc.Cf), k = pk1(kc.kf), U = pk1(Uf), e = pk1(kick);
+    return Quad{fma2(e, fma2(C, u.a, mul2(k, sub2(U, u.a))), p.a),
+                fma2(e, fma2(C, u.b, mul2(k, sub2(U, u.b))), p.b)};
+}
+__device__ __forceinline__ Quad quad_axpy(float d, const Quad &p, const Quad &x) {
+    const pair_t e = pk1(d);
+    return Quad{fma2(e, p.a, x.a), fma2(e, p.b, x.b)};
+}
+__device__ __forceinline__ Quad quad_sub(const Quad &a, const Quad &b) { return Quad{sub2(a.a, b.a), sub2(a.b, b.b)}; }
 
 // CTA-wide sums in FP32-pipe arithmetic (FP64 issues at a small fraction of
 // the FP32 rate on GB300), blockDim a multiple of 32 and at most 256.  The
@@ -292,12 +363,9 @@ __device__ void inf_pass(const FusedArgs &A, const PassCfg &pc, const InfConst &
         const int n = quad_len(i0, N);
         const Quad x = ldq<V4>(src, i0, N);
         const Quad t = quad_tanh(A, kc, x, Sf, i0, n);
-        Quad u;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) u.v[k] = t.v[k] - x.v[k];
-        su += quad_sum(u, n);
+        su += quad_sum(quad_sub(t, x), n);
         // the last pass's configuration is the proposal
-        if constexpr (LAST) quad_action(A, kc, x, t, Sdf, i0, n, pc.traj, A.seed, chain, tab, acc);
+        if constexpr (LAST) quad_action(A, kc, x, t, Sdf, i0, n, pc.traj, kc.rk, chain, tab, acc);
     }
     const float Uf = bsum_f32(su, red);
 
@@ -310,29 +378,17 @@ __device__ void inf_pass(const FusedArgs &A, const PassCfg &pc, const InfConst &
         const Quad t = quad_tanh(A, kc, x, Sf, i0, n);
         Quad pv;
         if constexpr (FIRST) {
-            const float4 w = momenta4_f32((uint32_t)q, pc.traj, (uint32_t)chain, A.seed);
-            pv.v[0] = w.x; pv.v[1] = w.y; pv.v[2] = w.z; pv.v[3] = w.w;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (k < n) acc_add(acc.K0, acc.K0lo, two_prod(pv.v[k], 0.5f * pv.v[k]));
+            pv = make_quad(momenta4((uint32_t)q, pc.traj, (uint32_t)chain, kc.rk));
+            quad_kinetic(pv, n, acc.K0, acc.K0lo);
         } else {
             pv = ldq<V4>(gp, i0, N);
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float u = t.v[k] - x.v[k];
-            const float F = fmaf(kc.Cf, u, kc.kf * (Uf - u));
-            pv.v[k] = fmaf(pc.kick, F, pv.v[k]);
-        }
+        pv = quad_kick(kc, pc.kick, pv, quad_sub(t, x), Uf);
         stq<V4>(gp, i0, N, pv);
         if constexpr (LAST) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (k < n) acc_add(acc.K1, acc.K1lo, two_prod(pv.v[k], 0.5f * pv.v[k]));
+            quad_kinetic(pv, n, acc.K1, acc.K1lo);
         } else {
-            Quad xn;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) xn.v[k] = fmaf(pc.drift, pv.v[k], x.v[k]);
+            const Quad xn = quad_axpy(pc.drift, pv, x);
             stq<V4>(dst, i0, N, xn);
             sp = df_add_f(sp, quad_sum(xn, n));
         }
@@ -345,7 +401,7 @@ __device__ void inf_pass(const FusedArgs &A, const PassCfg &pc, const InfConst &
 // flip proposal).
 template <bool V4>
 __device__ void inf_action(const FusedArgs &A, const InfConst &kc, int chain, int buf, float sign,
-                           uint32_t spin_traj, uint64_t seed, Red &red, const float4 *tab,
+                           uint32_t spin_traj, const uint32_t *seed, Red &red, const float4 *tab,
                            Acc &acc) {
     const int64_t N = A.g.N;
     const int64_t nq = (N + 3) >> 2;
@@ -358,8 +414,7 @@ __device__ void inf_action(const FusedArgs &A, const InfConst &kc, int chain, in
         const int64_t i0 = 4 * q;
         const int n = quad_len(i0, N);
         Quad v = ldq<V4>(x, i0, N);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v.v[k] *= sign;
+        if (sign < 0.0f) v = quad_neg(v);
         const Quad t = quad_tanh(A, kc, v, Sf, i0, n);
         quad_action(A, kc, v, t, Sdf, i0, n, spin_traj, seed, chain, tab, acc);
     }
@@ -501,7 +556,7 @@ __device__ __forceinline__ void res_pass(const FusedArgs &A, const InfConst &kc,
 #pragma unroll 1
         for (int k = 0; k < QPT; ++k) {
             const int64_t q = threadIdx.x + (int64_t)k * blockDim.x;
-            if (FULL || q < nq) aux[q] = momenta4_f32((uint32_t)q, traj, (uint32_t)chain, A.seed);
+            if (FULL || q < nq) aux[q] = momenta4((uint32_t)q, traj, (uint32_t)chain, kc.rk);
         }
     }
     float su = 0.0f;
@@ -514,15 +569,13 @@ __device__ __forceinline__ void res_pass(const FusedArgs &A, const InfConst &kc,
             const int64_t i0 = 4 * q;
             const int n = (FULL ? 4 : quad_len(i0, N));
             const Quad t = quad_tanh(A, kc, x[k], Sf, i0, n);
-            Quad u;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) u.v[e] = t.v[e] - x[k].v[e];
-            us[q] = make_float4(u.v[0], u.v[1], u.v[2], u.v[3]);
+            const Quad u = quad_sub(t, x[k]);
+            us[q] = to_float4(u);
             su += quad_sum(u, n);
             if constexpr (ONE_PASS)
-                quad_action(A, kc, x[k], t, Sdf, i0, n, traj, A.seed, chain, tab, acc);
+                quad_action(A, kc, x[k], t, Sdf, i0, n, traj, kc.rk, chain, tab, acc);
             else if constexpr (LAST)
-                aux[q] = make_float4(x[k].v[0], x[k].v[1], x[k].v[2], x[k].v[3]);
+                aux[q] = to_float4(x[k]);
         }
     }
     if constexpr (LAST && !ONE_PASS) {
@@ -534,10 +587,9 @@ __device__ __forceinline__ void res_pass(const FusedArgs &A, const InfConst &kc,
             if (FULL || q < nq) {
                 const int64_t i0 = 4 * q;
                 const int n = (FULL ? 4 : quad_len(i0, N));
-                const float4 w = aux[q];
-                const Quad xq{{w.x, w.y, w.z, w.w}};
+                const Quad xq = make_quad(aux[q]);
                 const Quad t = quad_tanh(A, kc, xq, Sf, i0, n);
-                quad_action(A, kc, xq, t, Sdf, i0, n, traj, A.seed, chain, tab, acc);
+                quad_action(A, kc, xq, t, Sdf, i0, n, traj, kc.rk, chain, tab, acc);
             }
         }
     }
@@ -549,27 +601,14 @@ __device__ __forceinline__ void res_pass(const FusedArgs &A, const InfConst &kc,
         if (FULL || q < nq) {
             const int n = (FULL ? 4 : quad_len(4 * q, N));
             if constexpr (FIRST) {
-                const float4 w = ONE_PASS ? momenta4_f32((uint32_t)q, traj, (uint32_t)chain, A.seed)
-                                          : aux[q];
-                pm[k].v[0] = w.x; pm[k].v[1] = w.y; pm[k].v[2] = w.z; pm[k].v[3] = w.w;
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (e < n) acc_add(acc.K0, acc.K0lo, two_prod(pm[k].v[e], 0.5f * pm[k].v[e]));
+                pm[k] = make_quad(ONE_PASS ? momenta4((uint32_t)q, traj, (uint32_t)chain, kc.rk) : aux[q]);
+                quad_kinetic(pm[k], n, acc.K0, acc.K0lo);
             }
-            const float4 u4 = us[q];
-            const float u[4] = {u4.x, u4.y, u4.z, u4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float F = fmaf(kc.Cf, u[e], kc.kf * (Uf - u[e]));
-                pm[k].v[e] = fmaf(kick, F, pm[k].v[e]);
-            }
+            pm[k] = quad_kick(kc, kick, pm[k], make_quad(us[q]), Uf);
             if constexpr (LAST) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (e < n) acc_add(acc.K1, acc.K1lo, two_prod(pm[k].v[e], 0.5f * pm[k].v[e]));
+                quad_kinetic(pm[k], n, acc.K1, acc.K1lo);
             } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) x[k].v[e] = fmaf(drift, pm[k].v[e], x[k].v[e]);
+                x[k] = quad_axpy(drift, pm[k], x[k]);
                 sp = df_add_f(sp, quad_sum(x[k], n));
             }
         }
@@ -608,7 +647,7 @@ __device__ void res_trajectories(const FusedArgs &A, const Schedule &S, const Ch
     const int64_t cbase = (int64_t)chain * N;
     Quad x[QPT], pm[QPT];
 #pragma unroll
-    for (int k = 0; k < QPT; ++k) x[k] = pm[k] = Quad{{0.0f, 0.0f, 0.0f, 0.0f}};
+    for (int k = 0; k < QPT; ++k) x[k] = pm[k] = Quad{0ull, 0ull};
     int start = st->start;
     res_load<V4, QPT, FULL>(sel3(A, start) + cbase, N, x);
     // sum of the current configuration (the order of chain_sum)
@@ -661,11 +700,9 @@ __device__ void res_trajectories(const FusedArgs &A, const Schedule &S, const Ch
                 if (FULL || q < nq) {
                     const int64_t i0 = 4 * q;
                     const int n = (FULL ? 4 : quad_len(i0, N));
-                    Quad v4 = x[k];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) v4.v[e] *= -1.0f;
+                    const Quad v4 = quad_neg(x[k]);
                     const Quad t = quad_tanh(A, kc, v4, Sf, i0, n);
-                    quad_action(A, kc, v4, t, Sdf, i0, n, traj, A.seed, chain, tab, fa);
+                    quad_action(A, kc, v4, t, Sdf, i0, n, traj, kc.rk, chain, tab, fa);
                 }
             }
             double w[5];
@@ -673,9 +710,7 @@ __device__ void res_trajectories(const FusedArgs &A, const Schedule &S, const Ch
             if (flip_decision(A, st, prm, chain, traj, w, invN, bcast)) {
                 const int f = (start != prop) ? 3 - start - prop : (start + 1) % 3;
 #pragma unroll
-                for (int k = 0; k < QPT; ++k)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) x[k].v[e] = -x[k].v[e];
+                for (int k = 0; k < QPT; ++k) x[k] = quad_neg(x[k]);
                 res_store<V4, QPT, FULL>(sel3(A, f) + cbase, N, x);
                 start = f;
                 Sstart = neg;
@@ -691,7 +726,8 @@ __device__ void res_trajectories(const FusedArgs &A, const Schedule &S, const Ch
 // thread's QPT quads inside the chain): the bounds and quad-length checks
 // fold away; the arithmetic and its order are those of the general instance.
 template <bool V4, int QPT, bool FULL = false>
-__global__ void __launch_bounds__(INF_MAX_THREADS, 2) infinite_kernel(FusedArgs A, Schedule S) {
+__global__ void __launch_bounds__(INF_MAX_THREADS, 2)
+    infinite_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ Schedule S) {
     __shared__ float4 tab_s[LOG1PEXP_NODES];
     __shared__ float red_f[16];
     __shared__ f2 red_d[64];
@@ -707,20 +743,21 @@ __global__ void __launch_bounds__(INF_MAX_THREADS, 2) infinite_kernel(FusedArgs 
     if (A.mode == MODE_MOMENTA) {
         float *gp = A.p + (int64_t)chain * N;
         for (int64_t q = threadIdx.x; q < ((N + 3) >> 2); q += blockDim.x) {
-            const float4 w = momenta4_f32((uint32_t)q, A.traj0, (uint32_t)chain, A.seed);
-            stq<V4>(gp, 4 * q, N, Quad{{w.x, w.y, w.z, w.w}});
+            stq<V4>(gp, 4 * q, N, make_quad(momenta4((uint32_t)q, A.traj0, (uint32_t)chain, A.round_keys)));
         }
         return;
     }
     for (int i = threadIdx.x; i < LOG1PEXP_NODES; i += blockDim.x) tab_s[i] = A.lpe_tab[i];
     __syncthreads();
-    const InfConst kc = inf_const(prm);
+    InfConst kc = inf_const(prm);
+    kc.rk = A.round_keys;
+    kc.rk0 = A.round_keys0;
     Red red{red_f, red_d, 0};
 
     if (A.mode == MODE_EVAL) {
         Acc acc = acc_zero();
         const int start = st->start;
-        inf_action<V4>(A, kc, chain, start, 1.0f, TRAJ_INIT, 0, red, tab_s, acc);
+        inf_action<V4>(A, kc, chain, start, 1.0f, TRAJ_INIT, kc.rk0, red, tab_s, acc);
         double v[5];
         action_totals(acc, v, red);
         if (threadIdx.x == 0) {
@@ -766,7 +803,7 @@ __global__ void __launch_bounds__(INF_MAX_THREADS, 2) infinite_kernel(FusedArgs 
         // ---- optional global sign flip psi -> -psi (Sec. 3, ergodicity) ----
         if (A.flip_every > 0 && ((traj + 1) % (uint32_t)A.flip_every) == 0) {
             Acc fa = acc_zero();
-            inf_action<V4>(A, kc, chain, start, -1.0f, traj, A.seed, red, tab_s, fa);
+            inf_action<V4>(A, kc, chain, start, -1.0f, traj, kc.rk, red, tab_s, fa);
             double w[5];
             action_totals(fa, w, red);
             if (flip_decision(A, st, prm, chain, traj, w, invN, bcast)) {
@@ -777,10 +814,7 @@ __global__ void __launch_bounds__(INF_MAX_THREADS, 2) infinite_kernel(FusedArgs 
                 const float *gs = sel3(A, start) + (int64_t)chain * N;
                 float *gf = sel3(A, f) + (int64_t)chain * N;
                 for (int64_t q = threadIdx.x; q < ((N + 3) >> 2); q += blockDim.x) {
-                    Quad v4 = ldq<V4>(gs, 4 * q, N);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) v4.v[e] = -v4.v[e];
-                    stq<V4>(gf, 4 * q, N, v4);
+                    stq<V4>(gf, 4 * q, N, quad_neg(ldq<V4>(gs, 4 * q, N)));
                 }
                 start = f;
                 Sstart = csum_neg(Sstart);   // negation is exact in every partial sum
