@@ -55,6 +55,7 @@ int fused_lattice_pick(const Geometry &g, int *threads, int *depth) {
 
 cudaError_t fused_lattice_node(const FusedArgs &a, int threads, int depth,
                                cudaKernelNodeParams *np, void **args) {
+    if (a.tiny && a.mode == MODE_TRAJ) return tiny_lattice_node(a, np, args);
     if (a.march && a.mode == MODE_TRAJ)
         return a.g.dim == 3 ? march3_lattice_node(a, np, args) : march_lattice_node(a, np, args);
     const int vec = (a.g.X % 4 == 0 && a.g.P % 4 == 0) ? 4 : 1;

@@ -68,6 +68,7 @@ struct FusedArgs {
     int eval_start;          // lattice kernel: evaluate S and the observables of the start
                              // configuration in the first trajectory's first pass
     int bulk;                // lattice kernel: stage planes by bulk copies (16-byte planes)
+    int tiny;                // trajectories by the on-chip kernel for small lattices
     int march;               // threads per slab of a marching kernel (0: another kernel)
     int *err;
 };
@@ -118,6 +119,10 @@ int fused_lattice_valid_split(const Geometry &g, int threads, int depth, int cs)
 // kernel-node parameters.
 int march_lattice_threads(const Geometry &g);
 cudaError_t march_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args);
+// On-chip kernel for small lattices (one CTA per chain): 1 if it is the one to
+// take this many chains of this geometry; its kernel-node parameters.
+int tiny_lattice_fits(const Geometry &g, int n_chains);
+cudaError_t tiny_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args);
 // The same in 3D (rows a multiple of four long; one CTA or a cluster per chain).
 int march3_lattice_threads(const Geometry &g);
 cudaError_t march3_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args);

@@ -386,8 +386,14 @@ static int use_march(const ising_hmc *h) {
     if (h->dim == 3) return march3_lattice_threads(h->g);
     return h->cs == 1 ? march_lattice_threads(h->g) : 0;
 }
+// Trajectories on the on-chip kernel for small lattices: neither a launch shape
+// nor a split was asked for.
+static int use_tiny(const ising_hmc *h) {
+    return is_fp32_lattice(h) && h->auto_shape && h->auto_split && h->cs == 1 &&
+           tiny_lattice_fits(h->g, h->n_chains);
+}
 // What of a handle, besides its shape and split, selects the kernel.
-static int kernel_choice(const ising_hmc *h) { return staging_bulk(h) | (use_march(h) ? 2 : 0) | (h->auto_split ? 4 : 0); }
+static int kernel_choice(const ising_hmc *h) { return staging_bulk(h) | (use_march(h) ? 2 : 0) | (h->auto_split ? 4 : 0) | (use_tiny(h) ? 8 : 0); }
 static FusedArgs fused_args(ising_hmc *h) {
     FusedArgs a{};
     for (int i = 0; i < 3; ++i) a.psi[i] = (float *)h->psi[i];
@@ -404,6 +410,7 @@ static FusedArgs fused_args(ising_hmc *h) {
     a.cs = is_fp32_lattice(h) ? h->cs : 1;
     a.bulk = staging_bulk(h);
     a.march = use_march(h);
+    a.tiny = use_tiny(h);
     a.err = h->d_err;
     return a;
 }
@@ -414,7 +421,7 @@ static FusedArgs fused_args(ising_hmc *h) {
 static FusedArgs trajectory_args(ising_hmc *h) {
     FusedArgs a = fused_args(h);
     a.mode = MODE_TRAJ;
-    if (a.march && h->dim == 3 && h->auto_split) a.cs = march3_lattice_split(h->g, h->n_chains);
+    if (a.march && !a.tiny && h->dim == 3 && h->auto_split) a.cs = march3_lattice_split(h->g, h->n_chains);
     return a;
 }
 
