@@ -171,8 +171,8 @@ def measured_peaks_all():
 
 STAGING_NAMES = {0: "auto", 1: "threads", 2: "bulk"}
 
-TRAFFIC_SOURCES = ("fused_lattice_impl.cuh", "fused_lattice_2d.cu", "df32.cuh",
-                   "device_common.cuh", "mbarrier.cuh")
+TRAFFIC_SOURCES = ("march_lattice.cuh", "march_lattice.cu", "pair.cuh", "df32.cuh",
+                   "device_common.cuh")
 
 
 def traffic_source_sha():
@@ -183,23 +183,28 @@ def traffic_source_sha():
     return hashlib.sha256(data).hexdigest()[:16]
 
 
-def traffic_record(kernel, workload, depth=None):
-    """DRAM bytes per launch from a committed ncu summary (for the launch's
-    ring depth where one was captured), if it matches the current kernel
-    source."""
+def traffic_record(kernel, workload):
+    """DRAM bytes per launch from a committed ncu summary, if it matches the
+    current kernel source."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(p) as f:
             d = json.load(f)
         rec = d.get(kernel, {}).get(workload)
         if rec and rec.get("source_sha") == traffic_source_sha():
-            by_depth = rec.get("bytes_per_launch_by_depth", {})
-            if depth is not None and str(depth) in by_depth:
-                return by_depth[str(depth)]
             return rec.get("bytes_per_launch")
     except (OSError, ValueError):
         pass
     return None
+
+
+def march_bytes_per_site(n_md):
+    """HBM bytes per site and leapfrog trajectory of the 2D marching kernel: psi
+    and p in and out once per sweep of three force evaluations; the first sweep
+    reads no p, the last one writes no psi (unless it takes in an evaluation
+    left over from the threes)."""
+    between = n_md + 1 - 2
+    return 12 + 16 * (between // 3) + (16 if between % 3 == 2 else 12)
 
 
 # ---------------------------------------------------------------- reference ----
@@ -451,15 +456,14 @@ def run_ours(args):
                               device="cuda")
 
     # dominant kernel: one launch = one trajectory of all chains of the largest lattice
-    alg_bytes = 16.0 * N_MD * big * big * n_chains
+    alg_bytes = float(march_bytes_per_site(N_MD)) * big * big * n_chains
     dur = float(np.mean(big_ms)) / 1e3
     peak, peak_kind = measured_peaks()
     achieved = alg_bytes / dur / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_source": peak_kind,
-                "traffic": traffic_record("fused_lattice_kernel", "2d_L%d_B%d" % (big, n_chains),
-                                          sims[big].launch[1]),
-                "kernel": "fused_lattice_kernel", "algorithmic_bytes_per_launch": alg_bytes,
+                "traffic": traffic_record("march_lattice_kernel", "2d_L%d_B%d" % (big, n_chains)),
+                "kernel": "march_lattice_kernel", "algorithmic_bytes_per_launch": alg_bytes,
                 "ms_per_launch": dur * 1e3}
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
@@ -1122,7 +1126,7 @@ def mixed_3d_rate(pkg, steps=4, seed=31):
                 "tuned_launch": tuned, "group_autotune_ms": group_ms, "acceptance": acc,
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                              "frac": achieved / peak, "peak_source": peak_kind,
-                             "kernel": "group graph (fused_lattice_kernel, five sizes)",
+                             "kernel": "group graph (march3_kernel, five sizes)",
                              "algorithmic_bytes_per_step": 16.0 * work / steps}}
     finally:
         grp.close()
