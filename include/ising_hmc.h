@@ -280,7 +280,10 @@ int ising_hmc_get_staging(const ising_hmc_t *h);
  * covers threads and depth at one CTA per chain, then chain splits of 2, 4
  * and 8 CTAs at the best thread count, then (if the plane staging is
  * ISING_STAGING_AUTO and the rows allow bulk copies) both staging modes at
- * the chosen shape, setting the faster one explicitly.  Allocates the
+ * the chosen shape, setting the faster one explicitly, all on the
+ * plane-streaming kernel; then the kernel the library picks by itself, which
+ * has no shape, in 3D with each chain split too.  If that one is fastest the
+ * handle stays on it and ising_hmc_get_launch keeps its values.  Allocates the
  * temporary handle; synchronises. */
 ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms);
 

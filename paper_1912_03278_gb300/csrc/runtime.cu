@@ -1594,11 +1594,21 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
             best = ms_mode[i];
         }
     }
-    // the marching kernels, where they take the lattice: no shape to choose,
-    // in 3D a split
-    bool march = false;
-    t->auto_shape = true;
+    // the library's own choice (a marching kernel or the on-chip one, which have
+    // no shape), then in 3D the marching kernel with each split
+    bool march = false, own = false;
+    t->auto_shape = t->auto_split = true;
     t->staging = h->staging;
+    t->cs = 1;
+    if (use_march(t) || use_tiny(t)) {
+        const double ms = time_trajectories(t, reps, e0, e1);
+        if (ms > 0 && ms < best) {
+            best = ms;
+            bc = 1;
+            march = own = true;
+        }
+    }
+    t->auto_split = false;
     for (int c : {1, 2, 4, 8}) {
         t->cs = c;
         if (!use_march(t) || (c > 1 && h->g.nplanes < 2 * c)) continue;
@@ -1607,6 +1617,7 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
             best = ms;
             bc = c;
             march = true;
+            own = false;
         }
     }
     cudaEventDestroy(e0);
@@ -1614,7 +1625,7 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
     ising_hmc_destroy(t);
     if (best_ms) *best_ms = best;
     h->auto_shape = march;
-    h->auto_split = false;
+    h->auto_split = own;
     if (march) {
         h->cs = bc;
         return ISING_OK;

@@ -67,6 +67,28 @@ def test_slabs_and_shared_ctas(L, kw, n_chains):
     assert np.abs(ra - rb).max() <= 1e-12 * 4 * L[0] * L[1]
 
 
+# warps a CTA's 256 threads do not divide into: two of 96 threads, one of 160
+@pytest.mark.parametrize("n_chains", [2, 700])
+@pytest.mark.parametrize("X", [300, 382, 600])
+def test_uneven_groups(X, n_chains):
+    a, b = _run((X, 50), False, n_chains=n_chains, n_md=4), _run((X, 50), True, n_chains=n_chains, n_md=4)
+    for x, y in zip(a[0], b[0]):
+        assert np.array_equal(x, y)
+    assert np.abs(a[1] - b[1]).max() <= 1e-12 * 4 * X * 50
+
+
+@pytest.mark.parametrize("L", [(16, 16), (64, 40)])
+def test_autotuned_handles_keep_their_results(L):
+    out = []
+    for tune in (False, True):
+        with pkg.IsingHMC(dim=2, L=L, beta=0.43, eps=0.2, n_md=4, n_chains=5) as s:
+            if tune:
+                s.autotune(reps=1)
+            s.trajectories(3, 9)
+            out.append(s.state())
+    assert np.array_equal(*out)
+
+
 def test_falls_back_where_it_does_not_fit():
     # too few rows, rows too long: the plane kernel, same results either way
     for L in ((64, 23), (1028, 24)):
