@@ -1059,7 +1059,11 @@ static ising_status run_trajectories(ising_hmc *h, int64_t n, uint64_t seed) {
             done += k;
         }
     } else {
-        const int k = std::min(h->n_chains, PLAIN_STREAMS);
+        // (a stream under capture keeps to itself: creating streams is no part of a graph)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        const bool single = cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess ||
+                            cap != cudaStreamCaptureStatusNone;
+        const int k = single ? 1 : std::min(h->n_chains, PLAIN_STREAMS);
         if (k > 1) {
             for (int i = 0; i < k; ++i) {
                 if (!h->side[i])
