@@ -235,7 +235,8 @@ ising_status ising_hmc_sync(ising_hmc_t *h);
  * to choose: in 2D (rows of at most 1024 sites, at least 24 rows, chains not
  * split) with several force evaluations per sweep, in 3D (rows a multiple of 4)
  * on as many CTAs per chain as ising_hmc_set_chain_split asked for or, if it
- * was not called, the library picks for the number of chains.  Their psi and p
+ * was not called, the library picks for the number of chains; small lattices of
+ * which no split was asked for stay on chip as a whole.  Their psi and p
  * are bit for bit those of the plane-streaming kernel below, which a call of
  * ising_hmc_set_launch selects (as does, in 2D, a split); the FP64 sums (action, energies, estimators) equal them to rounding
  * and depend on nothing but the handle.
