@@ -16,8 +16,9 @@
 //    registers for the whole trajectory; global memory is read once per
 //    launch (and after a rejection) and written once per trajectory (the
 //    proposal and the end momenta);
-//  * streaming (any N): psi and p are re-read from global memory every pass,
-//    sweep 2 recomputes u from psi with the identical instructions.
+//  * streaming (any N): psi and p are re-read every pass, the leading quads'
+//    from shared memory (struct Kept), the rest from global memory; sweep 2
+//    recomputes u from psi with the identical instructions.
 // Every sum adds the same per-quad partial sums in the same order in both,
 // and the thread count depends on N alone.  The last pass of a trajectory also evaluates the
 // proposal's action to FP64 accuracy in double-float arithmetic, the kinetic
@@ -27,8 +28,11 @@
 // The updates and the action run on pairs of sites in packed FP32 instructions
 // (pair.cuh: the scalar operations' bits): the resident kernel is bound by issue
 // (2432 chains of N = 4096: 0.50 -> 0.47 ms per call of one trajectory), the streaming
-// one by issue and latency (304 chains of N = 50001: 1.35 -> 1.14 ms).
+// one by issue and latency (304 chains of N = 50001: 1.35 -> 1.14 ms; with kept
+// quads 0.99).
 #include <cuda_runtime.h>
+
+#include <atomic>
 
 #include "df32.cuh"
 #include "device_common.cuh"
@@ -341,27 +345,54 @@ struct PassCfg {
     uint32_t traj;
 };
 
+// The streaming variant's quads that stay in shared memory through a
+// trajectory: psi of the thread's first nx quads, p of its first np, slot
+// k * nt + tid each (written and read by the owning thread only).  What bounds the
+// variant besides issue is the L2: every evaluation moves 20 B per site through
+// it, and two psi buffers and p of 304 chains of N = 50000 (183 MB) do not fit
+// into its 129 MB.  psi is kept before p (three of the five accesses against two), and the
+// passes after the first drift in place, which leaves one psi buffer in use.
+// Kernel, one trajectory of N_md = 10, ms: 304 chains of N = 50000 0.92 -> 0.64,
+// 50001 0.97 -> 0.85, 20000 0.225 -> 0.195.  Loading one quad ahead of its use as well
+// gains 3% at 50000 and loses 6% to 11% at 50001 and at N = 9000 to 20000: left out.
+struct Kept {
+    ulonglong2 *x, *p;
+    int nx, np;
+};
+__device__ __forceinline__ Quad lds_quad(const ulonglong2 &v) { return Quad{v.x, v.y}; }
+
 // One force evaluation.  cs: sum of the source configuration on entry, of
 // the drifted one on exit (unchanged by the last pass, which does not drift).
+// The first pass drifts from the current configuration into the proposal's
+// buffer, the later ones in place (src == dst: a thread overwrites only the
+// quad it has just read); kept quads reach the buffers in the last pass.
 template <bool V4, bool FIRST, bool LAST>
 __device__ void inf_pass(const FusedArgs &A, const PassCfg &pc, const InfConst &kc, int chain,
-                         CSum &cs, Red &red, const float4 *tab, Acc &acc) {
+                         const Kept &kp, CSum &cs, Red &red, const float4 *tab, Acc &acc) {
     const int64_t N = A.g.N;
     const int64_t nq = (N + 3) >> 2;
     const int64_t cbase = (int64_t)chain * N;
-    const float *__restrict__ src = sel3(A, pc.src) + cbase;
-    float *__restrict__ dst = sel3(A, pc.dst) + cbase;
-    float *__restrict__ gp = A.p + cbase;
+    const float *src = sel3(A, pc.src) + cbase;
+    float *dst = sel3(A, pc.dst) + cbase;
+    float *gp = A.p + cbase;
     const float Sf = cs.Sf;
 
     // ---- sweep 1: U = sum_i (tanh(A psi + h')_i - psi_i) ----
     float su = 0.0f;
     f2 Sdf{0.0f, 0.0f};
     if constexpr (LAST) Sdf = csum_exact(cs, red);
-    for (int64_t q = threadIdx.x; q < nq; q += blockDim.x) {
+    int k = 0;
+    for (int64_t q = threadIdx.x; q < nq; q += blockDim.x, ++k) {
         const int64_t i0 = 4 * q;
         const int n = quad_len(i0, N);
-        const Quad x = ldq<V4>(src, i0, N);
+        Quad x;
+        if (!FIRST && k < kp.nx) {
+            x = lds_quad(kp.x[q]);
+            if constexpr (LAST) stq<V4>(dst, i0, N, x);
+        } else {
+            x = ldq<V4>(src, i0, N);
+            if (FIRST && k < kp.nx) kp.x[q] = make_ulonglong2(x.a, x.b);
+        }
         const Quad t = quad_tanh(A, kc, x, Sf, i0, n);
         su += quad_sum(quad_sub(t, x), n);
         // the last pass's configuration is the proposal
@@ -371,25 +402,31 @@ __device__ void inf_pass(const FusedArgs &A, const PassCfg &pc, const InfConst &
 
     // ---- sweep 2: kick with F = A u, drift ----
     f2 sp{0.0f, 0.0f};
-    for (int64_t q = threadIdx.x; q < nq; q += blockDim.x) {
+    k = 0;
+    for (int64_t q = threadIdx.x; q < nq; q += blockDim.x, ++k) {
         const int64_t i0 = 4 * q;
         const int n = quad_len(i0, N);
-        const Quad x = ldq<V4>(src, i0, N);
-        const Quad t = quad_tanh(A, kc, x, Sf, i0, n);
-        Quad pv;
+        Quad x, pv;
+        if (k < kp.nx) x = lds_quad(kp.x[q]);
+        else x = ldq<V4>(src, i0, N);
         if constexpr (FIRST) {
             pv = make_quad(momenta4((uint32_t)q, pc.traj, (uint32_t)chain, kc.rk));
             quad_kinetic(pv, n, acc.K0, acc.K0lo);
+        } else if (k < kp.np) {
+            pv = lds_quad(kp.p[q]);
         } else {
             pv = ldq<V4>(gp, i0, N);
         }
+        const Quad t = quad_tanh(A, kc, x, Sf, i0, n);
         pv = quad_kick(kc, pc.kick, pv, quad_sub(t, x), Uf);
-        stq<V4>(gp, i0, N, pv);
+        if (!LAST && k < kp.np) kp.p[q] = make_ulonglong2(pv.a, pv.b);
+        else stq<V4>(gp, i0, N, pv);
         if constexpr (LAST) {
             quad_kinetic(pv, n, acc.K1, acc.K1lo);
         } else {
             const Quad xn = quad_axpy(pc.drift, pv, x);
-            stq<V4>(dst, i0, N, xn);
+            if (k < kp.nx) kp.x[q] = make_ulonglong2(xn.a, xn.b);
+            else stq<V4>(dst, i0, N, xn);
             sp = df_add_f(sp, quad_sum(xn, n));
         }
     }
@@ -772,6 +809,17 @@ __global__ void __launch_bounds__(INF_MAX_THREADS, 2)
         return;
     }
 
+    Kept kp;
+    {
+        uint32_t bytes;
+        asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(bytes));
+        const int slots = (int)(bytes / (sizeof(float4) * blockDim.x));
+        const int per = (int)((((N + 3) >> 2) + blockDim.x - 1) / blockDim.x);
+        kp.nx = min(slots, per);
+        kp.np = min(slots - kp.nx, per);
+        kp.x = reinterpret_cast<ulonglong2 *>(us);
+        kp.p = kp.x + (int64_t)kp.nx * blockDim.x;
+    }
     int start = st->start;
     // sum of the current configuration, carried from trajectory to trajectory
     CSum Sstart = chain_sum<V4>(sel3(A, start) + (int64_t)chain * N, N, red);
@@ -779,22 +827,22 @@ __global__ void __launch_bounds__(INF_MAX_THREADS, 2)
         const uint32_t traj = A.traj0 + (uint32_t)k;
         Acc acc = acc_zero();
         CSum cs = Sstart;
+        const int prop = buf_loc(start, S.n_pass - 1);
         // the integrator's force passes; the first draws the momenta (Sec. 3
         // refresh), the last evaluates the proposal's action
         for (int j = 0; j < S.n_pass; ++j) {
             PassCfg pc;
-            pc.src = buf_loc(start, j);
-            pc.dst = buf_loc(start, j + 1);
+            pc.src = j == 0 ? start : prop;
+            pc.dst = prop;
             pc.kick = (float)(S.kick[j] * prm.eps);
             pc.drift = (float)(S.drift[j] * prm.eps);
             pc.traj = traj;
             const bool first = j == 0, last = j == S.n_pass - 1;
-            if (first && last) inf_pass<V4, true, true>(A, pc, kc, chain, cs, red, tab_s, acc);
-            else if (first) inf_pass<V4, true, false>(A, pc, kc, chain, cs, red, tab_s, acc);
-            else if (last) inf_pass<V4, false, true>(A, pc, kc, chain, cs, red, tab_s, acc);
-            else inf_pass<V4, false, false>(A, pc, kc, chain, cs, red, tab_s, acc);
+            if (first && last) inf_pass<V4, true, true>(A, pc, kc, chain, kp, cs, red, tab_s, acc);
+            else if (first) inf_pass<V4, true, false>(A, pc, kc, chain, kp, cs, red, tab_s, acc);
+            else if (last) inf_pass<V4, false, true>(A, pc, kc, chain, kp, cs, red, tab_s, acc);
+            else inf_pass<V4, false, false>(A, pc, kc, chain, kp, cs, red, tab_s, acc);
         }
-        const int prop = buf_loc(start, S.n_pass - 1);
         double v[7];
         acc_totals(acc, v, red);
         const int cur = metropolis(A, st, prm, chain, traj, start, prop, v, invN, bcast);
@@ -860,26 +908,56 @@ static void *infinite_func(int qpt) {
     }
 }
 
+// Slots (a quad of every thread, 4 KB each) of the streaming variant's kept quads: what
+// fits beside the 19 KB of static arrays with two CTAs on an SM, or with one
+// where the launch has no second one for it.
+constexpr int INF_SLOTS_TWO = 23, INF_SLOTS_ONE = 51;
+constexpr size_t INF_SLOT_BYTES = INF_MAX_THREADS * sizeof(float4);
+constexpr size_t INF_STATIC_BYTES = LOG1PEXP_NODES * sizeof(float4) + 1024;
+static_assert(INF_SLOTS_TWO * INF_SLOT_BYTES + INF_STATIC_BYTES <= 113 * 1024, "two CTAs per SM");
+static_assert(INF_SLOTS_ONE * INF_SLOT_BYTES + INF_STATIC_BYTES <= 227 * 1024, "one CTA per SM");
+
+static size_t infinite_kept_bytes(int64_t N, int chains) {
+    static thread_local int sms = 0;
+    if (!sms) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            sms = 1;
+    }
+    const int64_t per = ((N + 3) / 4 + INF_MAX_THREADS - 1) / INF_MAX_THREADS;
+    const int64_t slots = chains <= sms ? INF_SLOTS_ONE : INF_SLOTS_TWO;
+    return (size_t)(slots < 2 * per ? slots : 2 * per) * INF_SLOT_BYTES;
+}
+
 cudaError_t infinite_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args) {
     const int qpt = infinite_qpt(a.g.N);
     const int64_t nq = (a.g.N + 3) / 4;
     const bool full = a.g.N % 4 == 0 && qpt > 0 && qpt <= 4 && nq == (int64_t)qpt * infinite_threads(a.g.N);
     np->func = full ? infinite_func<true, true>(qpt)
                     : (a.g.N % 4 == 0) ? infinite_func<true>(qpt) : infinite_func<false>(qpt);
-    static bool configured = false;   // room for the largest u and aux arrays above the static 20.5 KB
-    if (!configured) {
-        for (int q : {1, 2, 4, 8})
+    // room for the largest arrays above the static ones, once per device
+    static std::atomic<uint64_t> configured{0};
+    int dev = 0;
+    const cudaError_t ed = cudaGetDevice(&dev);
+    if (ed != cudaSuccess) return ed;
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if (!(configured.load() & bit)) {
+        for (int q : {0, 1, 2, 4, 8})
             for (void *f : {infinite_func<true>(q), infinite_func<false>(q), infinite_func<true, true>(q)}) {
                 const cudaError_t e = cudaFuncSetAttribute(
-                    f, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 8 * INF_MAX_THREADS * 16);
+                    f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                    q ? 2 * 8 * INF_MAX_THREADS * 16 : (int)(INF_SLOTS_ONE * INF_SLOT_BYTES));
                 if (e != cudaSuccess) return e;
             }
-        configured = true;
+        configured.fetch_or(bit);
     }
     np->gridDim = dim3((unsigned)(a.n_chains - a.chain0), 1, 1);
     np->blockDim = dim3((unsigned)infinite_threads(a.g.N), 1, 1);
-    // u and aux of the resident variant: at most 2 x 8 quads x 256 threads x 16 B = 64 KB
-    np->sharedMemBytes = (unsigned)(2 * qpt * infinite_threads(a.g.N) * sizeof(float4));
+    // u and aux of the resident variant: at most 2 x 8 quads x 256 threads x 16 B = 64 KB;
+    // the streaming variant's kept quads
+    np->sharedMemBytes = qpt ? (unsigned)(2 * qpt * infinite_threads(a.g.N) * sizeof(float4))
+                             : (unsigned)infinite_kept_bytes(a.g.N, a.n_chains - a.chain0);
     np->kernelParams = args;
     np->extra = nullptr;
     return cudaSuccess;
