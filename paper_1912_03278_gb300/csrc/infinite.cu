@@ -29,7 +29,7 @@
 // (pair.cuh: the scalar operations' bits): the resident kernel is bound by issue
 // (2432 chains of N = 4096: 0.50 -> 0.47 ms per call of one trajectory), the streaming
 // one by issue and latency (304 chains of N = 50001: 1.35 -> 1.14 ms; with kept
-// quads 0.99).
+// quads 1.00, with batched loads 0.78).
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -353,13 +353,43 @@ struct PassCfg {
 // into its 129 MB.  psi is kept before p (three of the five accesses against two), and the
 // passes after the first drift in place, which leaves one psi buffer in use.
 // Kernel, one trajectory of N_md = 10, ms: 304 chains of N = 50000 0.92 -> 0.64,
-// 50001 0.97 -> 0.85, 20000 0.225 -> 0.195.  Loading one quad ahead of its use as well
-// gains 3% at 50000 and loses 6% to 11% at 50001 and at N = 9000 to 20000: left out.
+// 50001 0.97 -> 0.85, 20000 0.225 -> 0.195.
 struct Kept {
     ulonglong2 *x, *p;
     int nx, np;
 };
 __device__ __forceinline__ Quad lds_quad(const ulonglong2 &v) { return Quad{v.x, v.y}; }
+
+// A quad inside the chain, without bounds checks.
+template <bool V4>
+__device__ __forceinline__ Quad ldq4(const float *p) {
+    if constexpr (V4) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
+        return Quad{t.x, t.y};
+    } else {
+        return make_quad(p[0], p[1], p[2], p[3]);
+    }
+}
+template <bool V4>
+__device__ __forceinline__ void stq4(float *p, const Quad &r) {
+    if constexpr (V4) {
+        *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(r.a, r.b);
+    } else {
+        float v[4];
+        unpack(r, v);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) p[k] = v[k];
+    }
+}
+
+// Quads per thread whose loads the middle passes issue together.  With 16 warps
+// on an SM the latency of the L2 bounded them (long-scoreboard stalls 1.36 per
+// issue at N = 20001), and the bounds checks of every quad kept loads from
+// being issued ahead.  One trajectory of N_md = 10, ms, without / 1 / 2 / 4 in a batch:
+// 304 chains of N = 50001 0.85 / 0.73 / 0.65 / 0.63, 50000 0.62 / 0.60 / 0.60 / 0.51, 20001
+// 0.250 / 0.234 / 0.219 / 0.225, 9000 0.102 / 0.100 / 0.100 / 0.097; 608 of 65536 1.84 / 1.75 / 1.74 /
+// 1.42; 152 of 200000 2.86 / 2.56 / 2.54 / 1.81.
+constexpr int INF_BATCH = 4;
 
 // One force evaluation.  cs: sum of the source configuration on entry, of
 // the drifted one on exit (unchanged by the last pass, which does not drift).
@@ -381,8 +411,21 @@ __device__ void inf_pass(const FusedArgs &A, const PassCfg &pc, const InfConst &
     float su = 0.0f;
     f2 Sdf{0.0f, 0.0f};
     if constexpr (LAST) Sdf = csum_exact(cs, red);
+    constexpr int NT = INF_MAX_THREADS;   // the block size of every chain that streams
+    // rows of whole quads, for which the middle passes need no bounds
+    const int rows = (FIRST || LAST) ? 0 : (int)(N / (4 * NT)) / INF_BATCH * INF_BATCH;
     int k = 0;
-    for (int64_t q = threadIdx.x; q < nq; q += blockDim.x, ++k) {
+    for (; k < rows; k += INF_BATCH) {
+        const int64_t q = threadIdx.x + (int64_t)k * NT;
+        Quad x[INF_BATCH];
+#pragma unroll
+        for (int b = 0; b < INF_BATCH; ++b)
+            x[b] = k + b < kp.nx ? lds_quad(kp.x[q + b * NT]) : ldq4<V4>(src + 4 * (q + b * NT));
+#pragma unroll
+        for (int b = 0; b < INF_BATCH; ++b)
+            su += quad_sum(quad_sub(quad_tanh(A, kc, x[b], Sf, 4 * (q + b * NT), 4), x[b]), 4);
+    }
+    for (int64_t q = threadIdx.x + (int64_t)k * NT; q < nq; q += NT, ++k) {
         const int64_t i0 = 4 * q;
         const int n = quad_len(i0, N);
         Quad x;
@@ -403,7 +446,27 @@ __device__ void inf_pass(const FusedArgs &A, const PassCfg &pc, const InfConst &
     // ---- sweep 2: kick with F = A u, drift ----
     f2 sp{0.0f, 0.0f};
     k = 0;
-    for (int64_t q = threadIdx.x; q < nq; q += blockDim.x, ++k) {
+    for (; k < rows; k += INF_BATCH) {
+        const int64_t q = threadIdx.x + (int64_t)k * NT;
+        Quad x[INF_BATCH], pv[INF_BATCH];
+#pragma unroll
+        for (int b = 0; b < INF_BATCH; ++b) {
+            x[b] = k + b < kp.nx ? lds_quad(kp.x[q + b * NT]) : ldq4<V4>(src + 4 * (q + b * NT));
+            pv[b] = k + b < kp.np ? lds_quad(kp.p[q + b * NT]) : ldq4<V4>(gp + 4 * (q + b * NT));
+        }
+#pragma unroll
+        for (int b = 0; b < INF_BATCH; ++b) {
+            const Quad t = quad_tanh(A, kc, x[b], Sf, 4 * (q + b * NT), 4);
+            pv[b] = quad_kick(kc, pc.kick, pv[b], quad_sub(t, x[b]), Uf);
+            x[b] = quad_axpy(pc.drift, pv[b], x[b]);
+            sp = df_add_f(sp, quad_sum(x[b], 4));
+            if (k + b < kp.np) kp.p[q + b * NT] = make_ulonglong2(pv[b].a, pv[b].b);
+            else stq4<V4>(gp + 4 * (q + b * NT), pv[b]);
+            if (k + b < kp.nx) kp.x[q + b * NT] = make_ulonglong2(x[b].a, x[b].b);
+            else stq4<V4>(dst + 4 * (q + b * NT), x[b]);
+        }
+    }
+    for (int64_t q = threadIdx.x + (int64_t)k * NT; q < nq; q += NT, ++k) {
         const int64_t i0 = 4 * q;
         const int n = quad_len(i0, N);
         Quad x, pv;
