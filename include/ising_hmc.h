@@ -181,11 +181,15 @@ ising_status ising_hmc_set_state(ising_hmc_t *h, const double *psi, int64_t next
 /* Same from a buffer in the state precision (FP64 for the plain form, FP32
  * otherwise), chain-major, in device memory or in (preferably pinned) host
  * memory: the copy uses unified addressing.  Bytes read:
- * n_chains*N*ising_hmc_state_elem_bytes(h). */
+ * n_chains*N*ising_hmc_state_elem_bytes(h).  Ordered after what the caller
+ * has queued on the default stream (and after the handle's own work); work on
+ * other streams that writes the buffer has to be complete. */
 ising_status ising_hmc_set_state_native(ising_hmc_t *h, const void *psi, int64_t next_traj);
 
 /* Copy the current configurations, in the state precision, to a device or
- * host buffer of n_chains*N elements.  Synchronises. */
+ * host buffer of n_chains*N elements.  Synchronises.  The buffer is written
+ * after what the caller has queued on the default stream; work on other
+ * streams that uses it has to be complete. */
 ising_status ising_hmc_get_state_native(ising_hmc_t *h, void *out);
 
 /* Bytes per state element: 8 (plain FP64 form) or 4. */

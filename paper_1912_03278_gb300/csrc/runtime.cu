@@ -71,6 +71,9 @@ struct ising_hmc {
     // the handle's stream (made at the first trajectory of several chains)
     cudaStream_t side[PLAIN_STREAMS] = {};
     cudaEvent_t fork = nullptr, join[PLAIN_STREAMS] = {};
+    // native copies: where the default stream of device caller_dev stood at the call
+    cudaEvent_t caller = nullptr;
+    int caller_dev = -1;
     double *series = nullptr;
     int64_t series_cap = 0, series_n = 0;
     // counters
@@ -310,6 +313,7 @@ static void free_all(ising_hmc *h) {
     for (auto &q : h->join)
         if (q) cudaEventDestroy(q);
     if (h->fork) cudaEventDestroy(h->fork);
+    if (h->caller) cudaEventDestroy(h->caller);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     h->stream = nullptr;
 }
@@ -1254,10 +1258,38 @@ ising_status ising_hmc_set_state(ising_hmc_t *h, const double *psi, int64_t next
     return after_set_state(h, next_traj);
 }
 
+// The caller's buffer may still be written or read by work it has queued on the
+// default stream, which the handle's (non-blocking) stream does not wait for by
+// itself: the handle's stream waits for it, on the device.  A handle whose stream is
+// being captured is refused before anything is queued (these calls synchronise).
+static cudaError_t after_default_stream(ising_hmc *h) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    for (cudaStream_t s : {h->stream, cudaStreamLegacy}) {
+        const cudaError_t e = cudaStreamIsCapturing(s, &cap);
+        if (e != cudaSuccess) return e;
+        if (cap != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
+    }
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && h->caller && h->caller_dev != dev) {
+        cudaEventDestroy(h->caller);
+        h->caller = nullptr;
+    }
+    if (e == cudaSuccess && !h->caller) {
+        e = cudaEventCreateWithFlags(&h->caller, cudaEventDisableTiming);
+        if (e != cudaSuccess) h->caller = nullptr;
+        h->caller_dev = dev;
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(h->caller, cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->caller, 0);
+    return e;
+}
+
 ising_status ising_hmc_set_state_native(ising_hmc_t *h, const void *psi_dev, int64_t next_traj) {
     NvtxRange nvtx_range("ising_hmc_set_state_native");
     if (!h || !psi_dev) return ISING_EINVAL;
     if (next_traj < 0 || next_traj > (int64_t)0xfffffffe) return fail(h, ISING_EINVAL, "bad trajectory index");
+    CUDA_OR_FAIL(h, after_default_stream(h));
     const size_t bytes = (size_t)h->n_chains * h->N * state_elem(h);
     // pinned (or mapped) host memory the device can read, 16-byte aligned:
     // the SMs copy it over the CPU-GPU link; anything else by cudaMemcpyAsync
@@ -1325,6 +1357,7 @@ ising_status ising_hmc_chain_params(const ising_hmc_t *h, double *out) {
 
 ising_status ising_hmc_get_state_native(ising_hmc_t *h, void *out) {
     if (!h || !out) return ISING_EINVAL;
+    CUDA_OR_FAIL(h, after_default_stream(h));
     const size_t cb = (size_t)h->N * state_elem(h);
     if (!is_fused(h)) {   // one buffer holds every chain
         CUDA_OR_FAIL(h, cudaMemcpyAsync(out, h->psi[0], cb * h->n_chains, cudaMemcpyDefault, h->stream));
