@@ -753,15 +753,17 @@ ising_status ising_mh_set_spins(ising_mh_t *h, const int8_t *in, int64_t next_sw
         if (in[i] != 1 && in[i] != -1) return mh_fail(h, ISING_EINVAL, "spin %zu is not +-1", i);
     ising_status st = ising_mh_sync(h);
     if (st != ISING_OK) return st;
+    // on the handle's stream, which a copy on the default stream is not ordered with
+    std::vector<uint32_t> w;
     if (h->packed) {
-        std::vector<uint32_t> w(n / 32, 0u);
+        w.assign(n / 32, 0u);
         for (size_t i = 0; i < n; ++i)
             if (in[i] > 0) w[i / 32] |= 1u << (i % 32);
-        if (cudaMemcpy(h->sw, w.data(), w.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess)
-            return mh_fail(h, ISING_ECUDA, "%s", cudaGetErrorString(cudaGetLastError()));
-    } else if (cudaMemcpy(h->s, in, n, cudaMemcpyHostToDevice) != cudaSuccess) {
-        return mh_fail(h, ISING_ECUDA, "%s", cudaGetErrorString(cudaGetLastError()));
     }
+    cudaError_t e = h->packed ? cudaMemcpyAsync(h->sw, w.data(), w.size() * 4, cudaMemcpyHostToDevice, h->stream)
+                              : cudaMemcpyAsync(h->s, in, n, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return mh_fail(h, ISING_ECUDA, "%s", cudaGetErrorString(e));
     h->sweep = next_sweep;
     return ISING_OK;
 }

@@ -1117,6 +1117,15 @@ static ising_status read_back(ising_hmc *h, void *dst, const void *src, size_t b
     return ISING_OK;
 }
 
+// Copies host memory to the handle's device memory and waits for it.  On the
+// handle's stream: the default stream, which a blocking copy runs on, is not ordered
+// with it (a copy from pageable memory may return before its last part has landed).
+static ising_status upload(ising_hmc *h, void *dst, const void *src, size_t bytes) {
+    CUDA_OR_FAIL(h, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, h->stream));
+    CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
+    return ISING_OK;
+}
+
 ising_status ising_hmc_sync(ising_hmc_t *h) {
     if (!h) return ISING_EINVAL;
     return read_back(h, nullptr, nullptr, 0);
@@ -1153,9 +1162,7 @@ ising_status ising_hmc_reset_sums(ising_hmc_t *h) {
     ising_status st = fetch_states(h, hs);
     if (st != ISING_OK) return st;
     for (auto &s : hs) std::memset(s.sums, 0, sizeof(s.sums));
-    CUDA_OR_FAIL(h, cudaMemcpy(h->d_state, hs.data(), sizeof(ChainState) * h->n_chains,
-                               cudaMemcpyHostToDevice));
-    return ISING_OK;
+    return upload(h, h->d_state, hs.data(), sizeof(ChainState) * h->n_chains);
 }
 
 ising_status ising_hmc_set_sums(ising_hmc_t *h, const double *in) {
@@ -1165,9 +1172,7 @@ ising_status ising_hmc_set_sums(ising_hmc_t *h, const double *in) {
     if (st != ISING_OK) return st;
     for (int c = 0; c < h->n_chains; ++c)
         std::memcpy(hs[c].sums, in + (size_t)c * ISING_NSUMS, sizeof(double) * ISING_NSUMS);
-    CUDA_OR_FAIL(h, cudaMemcpy(h->d_state, hs.data(), sizeof(ChainState) * h->n_chains,
-                               cudaMemcpyHostToDevice));
-    return ISING_OK;
+    return upload(h, h->d_state, hs.data(), sizeof(ChainState) * h->n_chains);
 }
 
 ising_status ising_hmc_observables(ising_hmc_t *h, ising_obs *out) {
@@ -1233,8 +1238,8 @@ static ising_status after_set_state(ising_hmc_t *h, int64_t next_traj) {
     ising_status st = fetch_states(h, hs);
     if (st != ISING_OK) return st;
     for (auto &s : hs) { s.start = 0; s.prop = 0; }
-    CUDA_OR_FAIL(h, cudaMemcpy(h->d_state, hs.data(), sizeof(ChainState) * h->n_chains,
-                               cudaMemcpyHostToDevice));
+    st = upload(h, h->d_state, hs.data(), sizeof(ChainState) * h->n_chains);
+    if (st != ISING_OK) return st;
     h->traj = next_traj;
     st = eval_current(h);
     if (st != ISING_OK) return st;
@@ -1249,12 +1254,13 @@ ising_status ising_hmc_set_state(ising_hmc_t *h, const double *psi, int64_t next
     if (st != ISING_OK) return st;
     const size_t total = (size_t)h->n_chains * h->N;
     if (state_elem(h) == sizeof(double)) {
-        CUDA_OR_FAIL(h, cudaMemcpy(h->psi[0], psi, total * sizeof(double), cudaMemcpyHostToDevice));
+        st = upload(h, h->psi[0], psi, total * sizeof(double));
     } else {
         std::vector<float> tmp(total);
         for (size_t i = 0; i < total; ++i) tmp[i] = (float)psi[i];
-        CUDA_OR_FAIL(h, cudaMemcpy(h->psi[0], tmp.data(), total * sizeof(float), cudaMemcpyHostToDevice));
+        st = upload(h, h->psi[0], tmp.data(), total * sizeof(float));
     }
+    if (st != ISING_OK) return st;
     return after_set_state(h, next_traj);
 }
 
@@ -2036,14 +2042,10 @@ ising_status ising_hmc_inject_device_error(ising_hmc_t *h, int bits) {
     if (bits & ~(KERR_TIMEOUT | KERR_BOUNDS)) return fail(h, ISING_EINVAL, "unknown error bits %d", bits);
     // OR into the word on the device, ordered after the handle's queued work
     int cur = 0;
-    ising_status st = ISING_OK;
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess ||
-        cudaMemcpy(&cur, h->d_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-        return fail(h, ISING_ECUDA, "inject: %s", cudaGetErrorString(cudaGetLastError()));
+    CUDA_OR_FAIL(h, cudaMemcpyAsync(&cur, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
     cur |= bits;
-    if (cudaMemcpy(h->d_err, &cur, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
-        st = fail(h, ISING_ECUDA, "inject: %s", cudaGetErrorString(cudaGetLastError()));
-    return st;
+    return upload(h, h->d_err, &cur, sizeof(int));
 }
 
 void ising_hmc_destroy(ising_hmc_t *h) {

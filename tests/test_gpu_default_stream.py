@@ -1,6 +1,7 @@
 """Native copies are ordered after work the caller has queued on the default
 stream, without a synchronise of the caller's: buffers that a kernel behind a
-long one still has to write (set) or overwrite (get)."""
+long one still has to write (set) or overwrite (get).  Uploads of host data are
+ordered with the handle's own work however busy the default stream is."""
 import numpy as np
 import pytest
 
@@ -56,3 +57,38 @@ def test_get_state_native_waits_for_the_default_stream(kind, where):
         pkg.ising_hmc_get_state_native(s.h, buf.data_ptr())
         torch.cuda.synchronize()
         assert np.array_equal(buf.cpu().double().numpy(), want)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_host_uploads_are_read_back_under_a_busy_default_stream(kind):
+    with pkg.IsingHMC(**KINDS[kind]) as s:
+        s.trajectories(2, 3)
+        sums = s.chain_sums() + 1.0
+        psi = workloads.start_psi(*s.state().shape, 1.0, seed=6)
+        if kind != "plain":
+            psi = psi.astype(np.float32).astype(np.float64)
+        _busy()
+        pkg.ising_hmc_set_sums(s.h, sums)
+        assert np.array_equal(s.chain_sums(), sums)
+        _busy()
+        s.set_state(psi, 4)
+        assert np.array_equal(s.state(), psi)
+        _busy()
+        pkg.ising_hmc_reset_sums(s.h)
+        assert not s.chain_sums().any()
+        _busy()
+        pkg.ising_hmc_inject_device_error(s.h, 1)
+        with pytest.raises(pkg.IsingError):
+            s.sync()
+
+
+@pytest.mark.parametrize("L", [(32, 8), (12, 8)])   # packed form, byte form
+def test_spins_are_read_back_under_a_busy_default_stream(L):
+    s = pkg.IsingMH(dim=2, L=L, beta=0.4, n_chains=3)
+    try:
+        spins = np.where(workloads.rng(8).random((3, L[0] * L[1])) < 0.5, -1, 1).astype(np.int8)
+        _busy()
+        s.set_spins(spins, next_sweep=2)
+        assert np.array_equal(s.spins(), spins)
+    finally:
+        s.close()
