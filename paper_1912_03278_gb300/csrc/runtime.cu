@@ -1230,9 +1230,11 @@ static ising_status after_set_state(ising_hmc_t *h, int64_t next_traj) {
         // current configuration in buffer 0; S and the observables come from
         // the first force pass of the next trajectory (no extra sweep)
         CUDA_OR_FAIL(h, launch_reset_chain_start(h->d_state, h->n_chains, h->stream));
+        const ising_status st = ising_hmc_sync(h);
+        if (st != ISING_OK) return st;   // (an earlier device error: the handle stays as it was)
         h->eval_pending = true;
         h->traj = next_traj;
-        return ising_hmc_sync(h);
+        return ISING_OK;
     }
     std::vector<ChainState> hs;
     ising_status st = fetch_states(h, hs);
