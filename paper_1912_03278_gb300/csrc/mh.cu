@@ -396,8 +396,9 @@ __global__ void __launch_bounds__(1024) mh_cluster_kernel(const __grid_constant_
             for (uint32_t w = cr * blockDim.x + threadIdx.x; w < nw; w += cs * blockDim.x)
                 packed_word<DIM, true>(a, sw, tt, w, chain, colour, 2 * (sweep0 + (uint32_t)k) + (uint32_t)colour,
                                        dM, dB, dF);
-            __syncwarp();
+            __syncwarp();   // (the loop's trip count differs between lanes)
             if (colour) add_sums(acc, dM, dB, dF);
+            __syncwarp();   // one lane added; the aligned barrier takes whole warps
             asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                          "barrier.cluster.wait.acquire.aligned;" ::: "memory");
         }

@@ -247,8 +247,10 @@ __device__ __forceinline__ uint32_t cluster_count() {
     asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r));
     return r;
 }
-// All threads of all CTAs of the cluster.
+// All threads of all CTAs of the cluster (the aligned form takes whole warps,
+// whose lanes may come from a branch of one of them).
 __device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n"
                  "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }

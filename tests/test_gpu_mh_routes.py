@@ -1,0 +1,39 @@
+"""The packed Metropolis-Hastings sweeps on each of their routes against the
+oracle, bit for bit; the number of launches tells which route ran."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1912_03278_gb300 as pkg
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(L, n_chains, calls, launches, n_therm=1, h=0.02):
+    betas = np.linspace(0.3, 0.6, n_chains)
+    sim = pkg.IsingMH(dim=len(L), L=L, beta=betas, h=h, n_chains=n_chains, n_therm=n_therm)
+    try:
+        got = []
+        for n in calls:
+            before = pkg.ising_mh_launch_count(sim.h)
+            sim.sweeps(n, 21)
+            got.append(pkg.ising_mh_launch_count(sim.h) - before)
+        assert got == launches
+        s, sums = sim.spins(), sim.chain_sums()
+    finally:
+        sim.close()
+    for c in range(n_chains):
+        model = oracle.Model(dim=len(L), L=L, beta=float(betas[c]), h=h, C=2 * len(L) * float(betas[c]) + 0.1)
+        rs, rsums = oracle.mh_checkerboard(model, seed=21, chain=c, n=sum(calls), n_therm=n_therm)
+        assert np.array_equal(s[c], rs) and np.array_equal(sums[c], rsums), c
+
+
+# a cluster per chain: warps whose lanes have different numbers of words, one to
+# eight CTAs
+@pytest.mark.parametrize("L", [(32, 6), (96, 70), (160, 122), (64, 12, 14)])
+def test_clusters(L):
+    _check(L, 3, [3, 2], [1, 1])
+
+
+def test_more_sweeps_than_a_launch_takes():
+    _check((32, 4), 2, [4099, 4], [2, 1], n_therm=4090)
