@@ -1023,14 +1023,10 @@ static int smem_with_table(K kern, int base, int threads) {
 
 template <int DIM, int VEC, int D, bool CL, bool BULK = false>
 cudaError_t kernel_node(const FusedArgs &a, int threads, cudaKernelNodeParams *np, void **args) {
-    static bool configured = false;
     auto kern = fused_lattice_kernel<DIM, VEC, D, CL, BULK>;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             227 * 1024);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e = allow_smem(once, kern, 227 * 1024);
+    if (e != cudaSuccess) return e;
     const int smem = smem_with_table(kern, (int)(ring_bytes(a.g.P, D) + RED_BYTES), threads);
     np->func = reinterpret_cast<void *>(kern);
     np->gridDim = dim3((unsigned)((a.n_chains - a.chain0) * a.cs), 1, 1);

@@ -32,8 +32,6 @@
 // quads 1.00, with batched loads 0.78).
 #include <cuda_runtime.h>
 
-#include <atomic>
-
 #include "df32.cuh"
 #include "device_common.cuh"
 #include "internal.h"
@@ -981,13 +979,7 @@ static_assert(INF_SLOTS_TWO * INF_SLOT_BYTES + INF_STATIC_BYTES <= 113 * 1024, "
 static_assert(INF_SLOTS_ONE * INF_SLOT_BYTES + INF_STATIC_BYTES <= 227 * 1024, "one CTA per SM");
 
 static size_t infinite_kept_bytes(int64_t N, int chains) {
-    static thread_local int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            sms = 1;
-    }
+    const int sms = sm_count();
     const int64_t per = ((N + 3) / 4 + INF_MAX_THREADS - 1) / INF_MAX_THREADS;
     const int64_t slots = chains <= sms ? INF_SLOTS_ONE : INF_SLOTS_TWO;
     return (size_t)(slots < 2 * per ? slots : 2 * per) * INF_SLOT_BYTES;
@@ -1000,12 +992,11 @@ cudaError_t infinite_node(const FusedArgs &a, cudaKernelNodeParams *np, void **a
     np->func = full ? infinite_func<true, true>(qpt)
                     : (a.g.N % 4 == 0) ? infinite_func<true>(qpt) : infinite_func<false>(qpt);
     // room for the largest arrays above the static ones, once per device
-    static std::atomic<uint64_t> configured{0};
+    static DeviceOnce once;
     int dev = 0;
     const cudaError_t ed = cudaGetDevice(&dev);
     if (ed != cudaSuccess) return ed;
-    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
-    if (!(configured.load() & bit)) {
+    const cudaError_t es = once.run(dev, [] {
         for (int q : {0, 1, 2, 4, 8})
             for (void *f : {infinite_func<true>(q), infinite_func<false>(q), infinite_func<true, true>(q)}) {
                 const cudaError_t e = cudaFuncSetAttribute(
@@ -1013,8 +1004,9 @@ cudaError_t infinite_node(const FusedArgs &a, cudaKernelNodeParams *np, void **a
                     q ? 2 * 8 * INF_MAX_THREADS * 16 : (int)(INF_SLOTS_ONE * INF_SLOT_BYTES));
                 if (e != cudaSuccess) return e;
             }
-        configured.fetch_or(bit);
-    }
+        return cudaSuccess;
+    });
+    if (es != cudaSuccess) return es;
     np->gridDim = dim3((unsigned)(a.n_chains - a.chain0), 1, 1);
     np->blockDim = dim3((unsigned)infinite_threads(a.g.N), 1, 1);
     // u and aux of the resident variant: at most 2 x 8 quads x 256 threads x 16 B = 64 KB;

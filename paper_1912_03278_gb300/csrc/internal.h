@@ -6,8 +6,33 @@
 #include <stdint.h>
 
 #include "../../include/ising_hmc.h"
+#include "device_once.h"
 
 namespace ihmc {
+
+// Lets launches of `kern` on the current device ask for up to `bytes` of dynamic
+// shared memory (the limit is per device); `once` is the kernel's own.
+template <class K>
+inline cudaError_t allow_smem(DeviceOnce &once, K kern, int bytes) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return once.run(dev, [&] {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    });
+}
+
+// SMs of the current device (1 if it gives no answer).
+inline int sm_count() {
+    static DeviceValue count;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    const int n = count.get(dev, [&] {
+        int v = 0;
+        return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? v : 0;
+    });
+    return n > 0 ? n : 1;
+}
 
 // Per-chain parameters (device).  hp = beta*h0 is the uniform part of h'.
 struct __align__(16) ChainParams {

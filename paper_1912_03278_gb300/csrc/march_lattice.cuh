@@ -743,13 +743,7 @@ struct Packing {
     int per_cta, slabs;
 };
 inline Packing pack_chains(int n_chains, int T, int rows) {
-    static thread_local int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            sms = 1;
-    }
+    const int sms = sm_count();
     const int most = MARCH_CTA_THREADS / T;
     int n = most;
     while (n > 1 && (n_chains + n - 1) / n < 2 * sms) --n;
@@ -762,13 +756,9 @@ inline Packing pack_chains(int n_chains, int T, int rows) {
 template <int TS, bool CUT, bool RAG, bool HF>
 cudaError_t node(const FusedArgs &a, int T, const Packing &pc, cudaKernelNodeParams *np, void **args) {
     auto kern = march_lattice_kernel<TS, CUT, MARCH_K, RAG, HF>;
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   227 * 1024);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e = allow_smem(once, kern, 227 * 1024);
+    if (e != cudaSuccess) return e;
     const int n = a.n_chains - a.chain0, groups = pc.per_cta * pc.slabs;
     np->func = reinterpret_cast<void *>(kern);
     np->gridDim = dim3((unsigned)((n + pc.per_cta - 1) / pc.per_cta), 1, 1);

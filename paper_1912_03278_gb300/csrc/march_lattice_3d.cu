@@ -15,13 +15,7 @@ int march3_lattice_threads(const Geometry &g) {
 // N_md = 10, at 1 / 2 / 4 CTAs per chain: L = 16 0.164 / 0.117 / 0.094 ms, 32
 // 0.281 / 0.187 / 0.145, 48 0.746 / 0.457 / 0.542, 64 1.358 / 0.780 / 0.934.
 int march3_lattice_split(const Geometry &g, int n_chains) {
-    static thread_local int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            sms = 1;
-    }
+    const int sms = sm_count();
     const int64_t T = m3_threads(g.X, g.Y);
     int cs = 1;
     while (cs < MAX_CS && g.nplanes >= 8 * cs &&

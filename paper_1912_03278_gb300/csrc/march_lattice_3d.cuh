@@ -400,13 +400,9 @@ __global__ void __launch_bounds__(M3_THREADS, 1)
 template <bool CL, bool HF, bool ODD>
 cudaError_t node3(const FusedArgs &a, cudaKernelNodeParams *np, void **args) {
     auto kern = march3_kernel<CL, HF, ODD>;
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   227 * 1024);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e = allow_smem(once, kern, 227 * 1024);
+    if (e != cudaSuccess) return e;
     np->func = reinterpret_cast<void *>(kern);
     np->gridDim = dim3((unsigned)((a.n_chains - a.chain0) * a.cs), 1, 1);
     np->blockDim = dim3((unsigned)a.march, 1, 1);

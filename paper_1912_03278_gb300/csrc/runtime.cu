@@ -1374,10 +1374,11 @@ ising_status ising_hmc_get_state_native(ising_hmc_t *h, void *out) {
     // memory of the GPU the handle's buffers are on: one gather launch;
     // anything else (host memory, another GPU) chain by chain
     cudaPointerAttributes pa{}, pm{};
-    const bool local = cudaPointerGetAttributes(&pa, out) == cudaSuccess &&
+    int dev = -1;   // (a launch needs the handle's GPU to be the current one)
+    const bool local = cudaPointerGetAttributes(&pa, out) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
                        cudaPointerGetAttributes(&pm, h->psi[0]) == cudaSuccess &&
                        pa.type == cudaMemoryTypeDevice && pm.type == cudaMemoryTypeDevice &&
-                       pa.device == pm.device && (uintptr_t)out % sizeof(float) == 0;
+                       pa.device == pm.device && pm.device == dev && (uintptr_t)out % sizeof(float) == 0;
     cudaGetLastError();
     if (local) {
         float *const psi[3] = {(float *)h->psi[0], (float *)h->psi[1], (float *)h->psi[2]};

@@ -249,13 +249,9 @@ __global__ void __launch_bounds__(TINY_THREADS)
 template <int DIM, int V, int QPT>
 cudaError_t tiny_node(const FusedArgs &a, int T, cudaKernelNodeParams *np, void **args) {
     auto kern = tiny_kernel<DIM, V, QPT>;
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   227 * 1024);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e = allow_smem(once, kern, 227 * 1024);
+    if (e != cudaSuccess) return e;
     const int N = (int)a.g.N, items = N / V;
     np->func = reinterpret_cast<void *>(kern);
     np->gridDim = dim3((unsigned)(a.n_chains - a.chain0), 1, 1);
@@ -289,14 +285,7 @@ int tiny_lattice_fits(const Geometry &g, int n_chains) {
     const bool v4 = g.X % 4 == 0 && g.P % 4 == 0;
     if ((g.dim != 2 && g.dim != 3) || g.N > (int64_t)TINY_THREADS * 4 * (v4 ? 4 : 1)) return 0;
     if (v4 ? g.N <= 1024 || (g.dim == 2 && g.X <= 32) : g.N <= 256) return 1;
-    static thread_local int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            sms = 1;
-    }
-    return n_chains <= 2 * sms;
+    return n_chains <= 2 * sm_count();
 }
 
 cudaError_t tiny_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args) {
