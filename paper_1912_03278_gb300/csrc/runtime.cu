@@ -1567,15 +1567,15 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
     if (reps < 1) reps = 1;
     ising_status st = ising_hmc_sync(h);
     if (st != ISING_OK) return st;
-    // temporary handle: same lattice and first chains' parameters, at most 2 waves of CTAs
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    // (more of short chains: several CTAs of few warps share an SM)
+    // temporary handle: same lattice and first chains' parameters, 2 CTAs per SM, and up
+    // to 8 of short chains (several CTAs of few warps share an SM) where that fits in memory
+    const int64_t nsm = sm_count();
     const int64_t most = std::min<int64_t>(8 * nsm, ((int64_t)1 << 28) / h->N);
-    const int nt = (int)std::min<int64_t>(h->n_chains, std::max<int64_t>(std::max(1, 2 * nsm), most));
+    const int least = (int)std::min<int64_t>(h->n_chains, 2 * nsm);
+    const int nt = (int)std::max<int64_t>(least, std::min<int64_t>(h->n_chains, most));
     ising_hmc *t = nullptr;
     st = clone_for_tuning(h, nt, &t);
+    if (st == ISING_ENOMEM && nt > least) st = clone_for_tuning(h, least, &t);
     if (st != ISING_OK) return fail(h, st, "autotune: %s", ising_hmc_last_create_error());
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
