@@ -1672,14 +1672,11 @@ ising_status ising_hmc_autotune(ising_hmc_t *h, int reps, double *best_ms) {
     if (best_ms) *best_ms = best;
     h->auto_shape = march;
     h->auto_split = own;
-    if (march) {
-        h->cs = bc;
-        return ISING_OK;
-    }
+    h->cs = bc;
+    h->staging = stg;   // (of the plane-streaming kernel, should a launch shape be set later)
+    if (march) return ISING_OK;
     h->threads = bt;
     h->depth = bd;
-    h->cs = bc;
-    h->staging = stg;
     return ISING_OK;
 }
 

@@ -29,3 +29,17 @@ def test_memory_that_suffices_for_no_temporary_handle_is_reported():
         finally:
             pkg.ising_hmc_inject_alloc_failure(0)
         assert ei.value.status == pkg.ISING_ENOMEM
+
+
+# a lattice for each kernel that can turn out fastest
+@pytest.mark.parametrize("kw", [dict(dim=2, L=(16, 16), n_chains=64), dict(dim=2, L=(128, 96), n_chains=320),
+                                dict(dim=3, L=(16, 16, 16), n_chains=64), dict(dim=3, L=(32, 32, 32), n_chains=160),
+                                dict(dim=2, L=(1028, 24), n_chains=3)])
+def test_settles_the_staging_whichever_kernel_is_fastest(kw):
+    with pkg.IsingHMC(beta=0.2, eps=0.1, n_md=4, **kw) as s:
+        s.autotune(reps=1)
+        assert s.staging in (pkg.ISING_STAGING_THREADS, pkg.ISING_STAGING_BULK)
+    with pkg.IsingHMC(beta=0.2, eps=0.1, n_md=4, **kw) as s:
+        s.set_staging(pkg.ISING_STAGING_THREADS)   # a choice of the caller's stays
+        s.autotune(reps=1)
+        assert s.staging == pkg.ISING_STAGING_THREADS
