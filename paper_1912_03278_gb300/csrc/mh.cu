@@ -3,19 +3,21 @@
 // the cost of a sweep against the cost of an HMC trajectory.
 //
 // Spins are int8 (+-1), chain-major, or, when rows are a multiple of 32 long,
-// packed 32 per word (multi-spin coding, mh_packed_kernel).  A sweep is three launches: colour 0,
-// colour 1 (c = (x + y + z) mod 2; with every extent even each bond joins the
-// two colours, so the sites of one colour see only the other colour and are
-// updated in parallel with the result of any sequential order), then a
-// per-chain step that turns the sweep's integer sums into observables.  A
-// thread owns 8 consecutive sites (group q; one 8-byte word when rows are a
-// multiple of 8 long), draws one Philox block per
-// half-sweep for the 4 of them that have its colour (site i uses word
-// (i/2) mod 4 of block i/8), and flips site i iff u23 < p, p from the chain's
-// FP32 table of min(1, exp(-2 beta s (J nb + h))) over s and the neighbour sum
-// nb.  The colour-0 launch adds its spins to the chain's spin sum M; the
-// colour-1 launch adds its spins and s_i * nb_i, which counts every bond once,
-// to M and the bond sum B (integers, exact in any order).
+// packed 32 per word (multi-spin coding).  A sweep updates colour 0, then colour 1
+// (c = (x + y + z) mod 2; with every extent even each bond joins the two colours, so
+// the sites of one colour see only the other colour and are updated in parallel
+// with the result of any sequential order), and turns the sweep's integer sums into
+// observables per chain.  The byte form takes three launches per sweep; the packed form runs
+// many sweeps per launch on a cluster of CTAs per chain (mh_cluster_kernel) or
+// two launches per sweep, each sweep measured by the next one's first
+// (mh_packed_kernel; the rule is in ising_mh_create).
+// In the byte form a thread owns 8 consecutive sites (group q; one 8-byte word when
+// rows are a multiple of 8 long), draws one Philox block per half-sweep for the 4 of
+// them that have its colour (site i uses word (i/2) mod 4 of block i/8), and flips
+// site i iff u23 < p, p from the chain's FP32 table of min(1, exp(-2 beta s (J nb +
+// h))) over s and the neighbour sum nb.  Colour 0 adds its spins to the chain's
+// spin sum M; colour 1 adds its spins and s_i * nb_i, which counts every bond
+// once, to M and the bond sum B (integers, exact in any order).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -37,3 +37,20 @@ def test_clusters(L):
 
 def test_more_sweeps_than_a_launch_takes():
     _check((32, 4), 2, [4099, 4], [2, 1], n_therm=4090)
+
+
+# a launch per colour: more chains than two CTAs per SM take in one wave, too few
+# words to fill two; the sums alternate between two sets, the next sweep's first
+# launch measures a sweep and a launch of its own the last one of a call
+@pytest.mark.parametrize("calls", [[3, 2], [1, 4], [2]])
+def test_a_launch_per_colour(calls):
+    import torch
+    n = 2 * torch.cuda.get_device_properties(0).multi_processor_count + 6
+    _check((32, 6), n, calls, [2 * k + 1 for k in calls])
+
+
+@pytest.mark.parametrize("L", [(64, 4, 6), (64,)])
+def test_a_launch_per_colour_in_other_dimensions(L):
+    import torch
+    n = 2 * torch.cuda.get_device_properties(0).multi_processor_count + 6
+    _check(L, n, [3], [7])
