@@ -266,6 +266,11 @@ ising_status ising_hmc_get_launch(const ising_hmc_t *h, int *threads, int *depth
 ising_status ising_hmc_set_chain_split(ising_hmc_t *h, int ctas);
 int ising_hmc_get_chain_split(const ising_hmc_t *h);
 
+/* Kernel that the next trajectories of an FP32 lattice handle run on, for tests
+ * and profiles; ISING_KERNEL_OTHER for the other forms. */
+enum { ISING_KERNEL_OTHER = 0, ISING_KERNEL_PLANE = 1, ISING_KERNEL_MARCH = 2, ISING_KERNEL_ONCHIP = 3 };
+int ising_hmc_trajectory_kernel(const ising_hmc_t *h);
+
 /* How the plane-streaming FP32 lattice kernel (see ising_hmc_set_launch) stages
  * psi and p planes into its shared-memory rings (Sec. 3's force evaluation streams the lattice plane by
  * plane): ISING_STAGING_THREADS, every thread copies its share of a plane

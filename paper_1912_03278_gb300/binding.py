@@ -19,6 +19,7 @@ LIB_PATH = os.path.join(HERE, "lib", "libising_hmc.so")
 # status codes
 ISING_OK, ISING_EINVAL, ISING_ENOTPD, ISING_ENOMEM, ISING_ECUDA, ISING_ETIMEOUT, ISING_EBUSY = range(7)
 ISING_STAGING_AUTO, ISING_STAGING_THREADS, ISING_STAGING_BULK = range(3)
+ISING_KERNEL_OTHER, ISING_KERNEL_PLANE, ISING_KERNEL_MARCH, ISING_KERNEL_ONCHIP = range(4)
 STATUS_NAMES = ["OK", "EINVAL", "ENOTPD", "ENOMEM", "ECUDA", "ETIMEOUT", "EBUSY"]
 ISING_KIND_LATTICE, ISING_KIND_DENSE, ISING_KIND_INFINITE = 0, 1, 2
 _KINDS = {"lattice": ISING_KIND_LATTICE, "dense": ISING_KIND_DENSE,
@@ -101,6 +102,7 @@ def load(path: str | None = None):
         "ising_hmc_autotune": (c_int, [P, c_int, P]),
         "ising_hmc_set_chain_split": (c_int, [P, c_int]),
         "ising_hmc_get_chain_split": (c_int, [P]),
+        "ising_hmc_trajectory_kernel": (c_int, [P]),
         "ising_hmc_set_staging": (c_int, [P, c_int]),
         "ising_hmc_get_staging": (c_int, [P]),
         "ising_group_autotune": (c_int, [P, c_int, P]),
@@ -379,6 +381,10 @@ def ising_hmc_get_chain_split(h) -> int:
 
 def ising_hmc_set_staging(h, mode):
     _check(h, load().ising_hmc_set_staging(h, int(mode)))
+
+
+def ising_hmc_trajectory_kernel(h) -> int:
+    return load().ising_hmc_trajectory_kernel(h)
 
 
 def ising_hmc_get_staging(h) -> int:
@@ -868,6 +874,11 @@ class IsingHMC:
     def set_staging(self, mode):
         """ISING_STAGING_AUTO, _THREADS or _BULK (FP32 lattice form)."""
         ising_hmc_set_staging(self.h, mode)
+
+    @property
+    def kernel(self):
+        """The kernel the next trajectories run on (FP32 lattice form)."""
+        return ising_hmc_trajectory_kernel(self.h)
 
     @property
     def staging(self):

@@ -1461,6 +1461,11 @@ ising_status ising_hmc_get_launch(const ising_hmc_t *h, int *threads, int *depth
     return ISING_OK;
 }
 
+int ising_hmc_trajectory_kernel(const ising_hmc_t *h) {
+    if (!h || !is_fp32_lattice(h)) return ISING_KERNEL_OTHER;
+    return use_tiny(h) ? ISING_KERNEL_ONCHIP : use_march(h) ? ISING_KERNEL_MARCH : ISING_KERNEL_PLANE;
+}
+
 ising_status ising_hmc_set_chain_split(ising_hmc_t *h, int ctas) {
     if (!h) return ISING_EINVAL;
     if (!is_fp32_lattice(h)) return fail(h, ISING_EINVAL, "chain split applies to the FP32 lattice form");
