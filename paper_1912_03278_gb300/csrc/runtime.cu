@@ -1117,11 +1117,17 @@ static ising_status read_back(ising_hmc *h, void *dst, const void *src, size_t b
     return ISING_OK;
 }
 
-// Copies host memory to the handle's device memory and waits for it.  On the
-// handle's stream: the default stream, which a blocking copy runs on, is not ordered
-// with it (a copy from pageable memory may return before its last part has landed).
-static ising_status upload(ising_hmc *h, void *dst, const void *src, size_t bytes) {
+// Queues a copy of host memory to the handle's device memory on the handle's stream:
+// the default stream, which a blocking copy runs on, is not ordered with it (a
+// copy from pageable memory may return before its last part has landed).  The
+// caller keeps `src` until it has waited for the stream.
+static ising_status queue_upload(ising_hmc *h, void *dst, const void *src, size_t bytes) {
     CUDA_OR_FAIL(h, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, h->stream));
+    return ISING_OK;
+}
+static ising_status upload(ising_hmc *h, void *dst, const void *src, size_t bytes) {
+    const ising_status st = queue_upload(h, dst, src, bytes);
+    if (st != ISING_OK) return st;
     CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
     return ISING_OK;
 }
@@ -1240,12 +1246,13 @@ static ising_status after_set_state(ising_hmc_t *h, int64_t next_traj) {
     ising_status st = fetch_states(h, hs);
     if (st != ISING_OK) return st;
     for (auto &s : hs) { s.start = 0; s.prop = 0; }
-    st = upload(h, h->d_state, hs.data(), sizeof(ChainState) * h->n_chains);
-    if (st != ISING_OK) return st;
-    h->traj = next_traj;
-    st = eval_current(h);
-    if (st != ISING_OK) return st;
-    return ising_hmc_sync(h);
+    st = queue_upload(h, h->d_state, hs.data(), sizeof(ChainState) * h->n_chains);
+    if (st == ISING_OK) {
+        h->traj = next_traj;
+        st = eval_current(h);
+    }
+    const ising_status waited = ising_hmc_sync(h);   // also after a failure: hs was queued
+    return st != ISING_OK ? st : waited;
 }
 
 ising_status ising_hmc_set_state(ising_hmc_t *h, const double *psi, int64_t next_traj) {
@@ -1255,15 +1262,17 @@ ising_status ising_hmc_set_state(ising_hmc_t *h, const double *psi, int64_t next
     ising_status st = ising_hmc_sync(h);
     if (st != ISING_OK) return st;
     const size_t total = (size_t)h->n_chains * h->N;
+    std::vector<float> tmp;
     if (state_elem(h) == sizeof(double)) {
-        st = upload(h, h->psi[0], psi, total * sizeof(double));
+        st = queue_upload(h, h->psi[0], psi, total * sizeof(double));
     } else {
-        std::vector<float> tmp(total);
+        tmp.resize(total);
         for (size_t i = 0; i < total; ++i) tmp[i] = (float)psi[i];
-        st = upload(h, h->psi[0], tmp.data(), total * sizeof(float));
+        st = queue_upload(h, h->psi[0], tmp.data(), total * sizeof(float));
     }
-    if (st != ISING_OK) return st;
-    return after_set_state(h, next_traj);
+    if (st == ISING_OK) st = after_set_state(h, next_traj);
+    if (st != ISING_OK) cudaStreamSynchronize(h->stream);   // (a success has waited)
+    return st;
 }
 
 // The caller's buffer may still be written or read by work it has queued on the
