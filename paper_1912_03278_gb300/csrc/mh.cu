@@ -41,6 +41,7 @@ constexpr uint32_t PURPOSE_MH = 5;
 constexpr int MH_THREADS = 256;
 constexpr int MH_TAB = 13;   // neighbour sums -6..6
 constexpr int64_t MH_CLUSTER_WORDS = 4096;   // words per SM up to which sweeps run on clusters
+constexpr int64_t MH_HOST_UNPACK_WORDS = 5120;
 
 // Per-chain parameters and sums.
 struct MHChain {
@@ -713,13 +714,14 @@ ising_status ising_mh_get_spins(ising_mh_t *h, int8_t *out) {
     ising_status st = ising_mh_sync(h);
     if (st != ISING_OK) return st;
     if (h->packed) {
-        // unpacked on the device, up to 64 MB at a time (the host's loop over
-        // the bits took about 1 ns per spin)
+        // Few words are copied and unpacked on the host, more on the device, up to 64 MB
+        // at a time.  Host / device: 6144 spins 15 / 28 us a call, 131072 30 / 32, 262144
+        // 43 / 33, 4 million 440 / 117.
         const int64_t nw = (int64_t)h->n_chains * (h->N / 32);
         const int64_t step = std::min<int64_t>(nw, (int64_t)1 << 21);
         void *buf = nullptr;
-        if (cudaMallocAsync(&buf, (size_t)step * 32, h->stream) != cudaSuccess) {
-            cudaGetLastError();   // no room: on the host
+        if (nw <= MH_HOST_UNPACK_WORDS || cudaMallocAsync(&buf, (size_t)step * 32, h->stream) != cudaSuccess) {
+            cudaGetLastError();   // (or no room)
             std::vector<uint32_t> w(nw);
             if (cudaMemcpy(w.data(), h->sw, (size_t)nw * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
                 return mh_fail(h, ISING_ECUDA, "%s", cudaGetErrorString(cudaGetLastError()));

@@ -54,3 +54,17 @@ def test_a_launch_per_colour_in_other_dimensions(L):
     import torch
     n = 2 * torch.cuda.get_device_properties(0).multi_processor_count + 6
     _check(L, n, [3], [7])
+
+
+# few spins are unpacked on the host, more by a launch
+@pytest.mark.parametrize("L,n_chains,launches", [((32, 6), 1, 0), ((64, 80), 32, 0), ((64, 80), 33, 1), ((128, 64), 40, 1)])
+def test_spins_unpacked_on_either_side(L, n_chains, launches):
+    sim = pkg.IsingMH(dim=2, L=L, beta=0.4, n_chains=n_chains)
+    try:
+        want = np.where(np.random.default_rng(3).random((n_chains, L[0] * L[1])) < 0.5, -1, 1).astype(np.int8)
+        sim.set_spins(want, next_sweep=0)
+        before = pkg.ising_mh_launch_count(sim.h)
+        assert np.array_equal(sim.spins(), want)
+        assert pkg.ising_mh_launch_count(sim.h) - before == launches
+    finally:
+        sim.close()
