@@ -56,6 +56,14 @@ def test_a_launch_per_colour_in_other_dimensions(L):
     _check(L, n, [3], [7])
 
 
+# more clusters than fit at once: small chains stay on them, longer ones take a
+# launch per colour
+@pytest.mark.parametrize("L,launches", [((64, 8), 1), ((128, 66), 7)])
+def test_several_waves_of_clusters(L, launches):
+    import torch
+    _check(L, 4 * torch.cuda.get_device_properties(0).multi_processor_count, [3], [launches])
+
+
 # few spins are unpacked on the host, more by a launch
 @pytest.mark.parametrize("L,n_chains,launches", [((32, 6), 1, 0), ((64, 80), 32, 0), ((64, 80), 33, 1), ((128, 64), 40, 1)])
 def test_spins_unpacked_on_either_side(L, n_chains, launches):
