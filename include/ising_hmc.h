@@ -234,16 +234,19 @@ int64_t ising_hmc_launch_count(const ising_hmc_t *h);
 /* Synchronise the handle's stream; ETIMEOUT if a device wait gave up. */
 ising_status ising_hmc_sync(ising_hmc_t *h);
 
-/* Lattices whose launch shape was left to the library run on
- * kernels that march through the planes with register windows and have no shape
- * to choose: in 2D (rows of at most 1024 sites, at least 24 rows, chains not
- * split) with several force evaluations per sweep, in 3D (rows a multiple of 4)
- * on as many CTAs per chain as ising_hmc_set_chain_split asked for or, if it
- * was not called, the library picks for the number of chains; small lattices of
- * which no split was asked for stay on chip as a whole.  Their psi and p
- * are bit for bit those of the plane-streaming kernel below, which a call of
- * ising_hmc_set_launch selects (as does, in 2D, a split); the FP64 sums (action, energies, estimators) equal them to rounding
- * and depend on nothing but the handle.
+/* FP32 lattices whose launch shape and chain split were left to the library run
+ * on the kernel that is fastest for their extents, number of chains, force
+ * evaluations per trajectory and field: small lattices on chip as a whole; 2D
+ * lattices (rows of at most 1024 sites, at least 24 rows) on a kernel that marches
+ * down the rows with several force evaluations per sweep; 3D ones (rows a
+ * multiple of 4) on one that marches through the planes, on as many CTAs per chain
+ * as the library picks; else on the plane-streaming kernel below.
+ * ising_hmc_set_launch selects the plane-streaming kernel.
+ * ising_hmc_set_chain_split selects, without a launch shape, the marching kernel
+ * where it takes the lattice: in 3D on that many CTAs per chain, in 2D for a
+ * split of 1 (other splits: plane-streaming).  psi and p are bit for bit the same
+ * on all of them; the FP64 sums (action, energies, estimators) equal one another to
+ * rounding and depend on nothing but the handle.
  *
  * Launch shape of the fused FP32 lattice kernel: threads per CTA (a multiple
  * of 32, at most 4 float4 vectors of a plane per thread; 32..256 with one CTA

@@ -143,16 +143,21 @@ int fused_lattice_valid_split(const Geometry &g, int threads, int depth, int cs)
 // threads per chain for this geometry (0 if it does not take it); its
 // kernel-node parameters.
 int march_lattice_threads(const Geometry &g);
+// 1 where it is faster than the plane-streaming kernel: this many chains, force
+// evaluations per trajectory, a field per site or not.
+int march_lattice_pays(const Geometry &g, int n_chains, int n_pass, bool field);
 cudaError_t march_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args);
 // On-chip kernel for small lattices (one CTA per chain): 1 if it is the one to
-// take this many chains of this geometry; its kernel-node parameters.
-int tiny_lattice_fits(const Geometry &g, int n_chains);
+// take this many chains of this geometry, n_pass force evaluations each; its kernel-node
+// parameters.
+int tiny_lattice_fits(const Geometry &g, int n_chains, int n_pass);
 cudaError_t tiny_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args);
 // The same in 3D (rows a multiple of four long; one CTA or a cluster per chain).
 int march3_lattice_threads(const Geometry &g);
 cudaError_t march3_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args);
 // CTAs per chain for a launch of this many chains when none was asked for.
 int march3_lattice_split(const Geometry &g, int n_chains);
+int march3_lattice_pays(const Geometry &g, int n_chains, int n_pass, bool field);
 // Cluster size of a graph kernel node made from fused_lattice_node (cs > 1).
 cudaError_t fused_lattice_node_cluster(cudaGraphNode_t node, int cs);
 int fused_lattice_pick(const Geometry &g, int *threads, int *depth);

@@ -1,4 +1,6 @@
 // march_lattice_3d.cu -- instances of march_lattice_3d.cuh without a field per site.
+#include <algorithm>
+
 #include "march_lattice_3d.cuh"
 
 namespace ihmc {
@@ -9,19 +11,49 @@ int march3_lattice_threads(const Geometry &g) {
     return T <= M3_THREADS && m3_smem(g.P, T) <= 227 * 1024 ? T : 0;
 }
 
+// CTAs resident on an SM: by threads (128 registers each) and shared memory.
+static int march3_resident(const Geometry &g) {
+    const int T = m3_threads(g.X, g.Y);
+    return std::min(M3_THREADS / T, (int)(227 * 1024 / (m3_smem(g.P, T) + 1024)));
+}
+
 // Chains are split while that leaves at most one CTA per SM, or CTAs so small
-// that their threads number below 352 per SM, each with four planes at least
-// (four more than its own are computed per evaluation).  Trajectories of 64 chains,
-// N_md = 10, at 1 / 2 / 4 CTAs per chain: L = 16 0.164 / 0.117 / 0.094 ms, 32
-// 0.281 / 0.187 / 0.145, 48 0.746 / 0.457 / 0.542, 64 1.358 / 0.780 / 0.934.
+// that their threads number at most 352 per SM, each with four planes at least
+// (four more than its own are computed per evaluation), and all are resident at
+// once, six at most on an SM.  Trajectories of 64 chains, N_md = 10, at 1 / 2 / 4 CTAs per
+// chain: L = 16 0.164 / 0.117 / 0.094 ms, 32 0.281 / 0.187 / 0.145, 48 0.746 / 0.457 / 0.542, 64
+// 1.358 / 0.780 / 0.934.  Against the plane-streaming kernel's time, nine evaluations: 200 chains of
+// 32^3 (337 threads per SM once split) 0.70 / 0.54, of 28^3 0.80 / 0.63; 400 chains of 20^3 0.97 /
+// 1.25 (five CTAs fit), of 16^3 0.92 / 0.80 / 1.12 (six); 304 chains of 8 x 8 x 20 0.96 / 0.69 /
+// 1.03 (eight).
 int march3_lattice_split(const Geometry &g, int n_chains) {
-    const int sms = sm_count();
-    const int64_t T = m3_threads(g.X, g.Y);
+    const int64_t T = m3_threads(g.X, g.Y), sms = sm_count(), n = n_chains;
+    const int64_t fit = sms * std::min(march3_resident(g), 6);
     int cs = 1;
-    while (cs < MAX_CS && g.nplanes >= 8 * cs &&
-           (2 * cs * (int64_t)n_chains <= sms || 2 * cs * n_chains * T <= 352 * (int64_t)sms))
+    while (cs < MAX_CS && g.nplanes >= 8 * cs && 2 * cs * n <= fit &&
+           (2 * cs * n <= sms || 2 * cs * n * T <= 352 * sms))
         cs *= 2;
     return cs;
+}
+
+// Planes of few tiles leave its CTAs with one or two warps and few of those fit on an
+// SM, so many such chains, and a field's loads, which nothing hides, are the
+// plane-streaming kernel's.  Against its time, nine evaluations (with a field per site):
+// 152 chains of 24^3 0.71 (0.89), 304 of 20^3 0.89 (1.00), of 24^3 0.91 (1.11), of 32^3 0.82 (0.98), 1000 of
+// 16^3 1.18 (1.54), of 12^3 0.90 (1.10), of 8 x 8 x 20 1.11 (1.30), of 20^3 0.97 (1.23), of 28^3 0.82
+// (1.05), of 32 x 32 x 16 0.65 (0.87); two evaluations, 304 of 24^3 1.11 (1.30).  Of fewer than
+// eight planes the four extra ones of every evaluation eat the gain (348 drawn lattices
+// 0.96 in the mean, a third of them slower).  With this rule one of 1750 lattices is
+// slower by more than 3 % (by 4).
+int march3_lattice_pays(const Geometry &g, int n_chains, int n_pass, bool field) {
+    const int T = m3_threads(g.X, g.Y), tiles = (g.X / 4) * ((g.Y + 1) / 2);
+    const int sms = sm_count(), per_sm = (n_chains + sms - 1) / sms, cs = march3_lattice_split(g, n_chains);
+    const bool longer = n_pass >= 9;
+    if (g.nplanes < 8) return 0;
+    if (T >= 256 || cs >= 4) return 1;
+    if (!field) return T >= 128 || per_sm == 1 || (longer && (T >= 96 || per_sm <= 3 || (T == 64 && tiles == T)));
+    if (T >= 128) return (per_sm == 1 && (longer || T >= 192)) || (longer && 8 * tiles >= 7 * T);
+    return longer && cs >= 2 && per_sm <= 2 && (T >= 64 || g.nplanes >= 16);
 }
 
 cudaError_t march3_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args) {

@@ -53,7 +53,7 @@ struct ising_hmc {
     // no launch shape asked for: the library may run trajectories on the
     // marching kernel, which has one shape per lattice
     bool auto_shape = true;
-    bool auto_split = true;   // no split asked for: the 3D marching kernel chooses one
+    bool auto_split = true;   // no split asked for: the library chooses (kernel, 3D split)
     // FP32 lattice form: the configurations were set from outside and their
     // action is evaluated by the next trajectory's first force pass
     bool eval_pending = false;
@@ -400,17 +400,20 @@ static int staging_bulk(const ising_hmc *h) {
 
 // Trajectories on a marching kernel -- 2D chains on one CTA each, 3D chains on
 // one CTA or a cluster -- unless a launch shape (a choice of the plane-streaming
-// kernel) was asked for.  The kernel's threads, 0 for the plane-streaming kernel.
+// kernel) was asked for, and, where no split was asked for either, if it is the
+// faster one.  The kernel's threads, 0 for the plane-streaming kernel.
 static int use_march(const ising_hmc *h) {
-    if (!is_fp32_lattice(h) || !h->auto_shape) return 0;
-    if (h->dim == 3) return march3_lattice_threads(h->g);
-    return h->cs == 1 ? march_lattice_threads(h->g) : 0;
+    if (!is_fp32_lattice(h) || !h->auto_shape || (h->dim != 3 && h->cs != 1)) return 0;
+    const int T = h->dim == 3 ? march3_lattice_threads(h->g) : march_lattice_threads(h->g);
+    if (!T || !h->auto_split) return T;
+    auto pays = h->dim == 3 ? march3_lattice_pays : march_lattice_pays;
+    return pays(h->g, h->n_chains, h->sched.n_pass, h->has_h) ? T : 0;
 }
 // Trajectories on the on-chip kernel for small lattices: neither a launch shape
 // nor a split was asked for.
 static int use_tiny(const ising_hmc *h) {
     return is_fp32_lattice(h) && h->auto_shape && h->auto_split && h->cs == 1 &&
-           tiny_lattice_fits(h->g, h->n_chains);
+           tiny_lattice_fits(h->g, h->n_chains, h->sched.n_pass);
 }
 // What of a handle, besides its shape and split, selects the kernel.
 static int kernel_choice(const ising_hmc *h) { return staging_bulk(h) | (use_march(h) ? 2 : 0) | (h->auto_split ? 4 : 0) | (use_tiny(h) ? 8 : 0); }

@@ -275,17 +275,30 @@ cudaError_t tiny_qpt(const FusedArgs &a, cudaKernelNodeParams *np, void **args) 
 
 }  // namespace
 
-// Few chains (two CTAs per SM at most): the latency of an evaluation counts and
-// the streaming kernels' is higher throughout (us per trajectory of 64 chains,
-// N_md = 8, here / there: 16 x 16 13 / 115, 31 x 33 42 / 182, 64 x 64 50 / 98, 512 x 16
-// 62 / 120, 16^3 52 / 62; 304 chains of 64 x 64 100 / 100).  Many chains: only where
-// the streaming kernels leave lanes idle (4096 chains: 16 x 16 93 / 371, 32 x 32 401 /
-// 412, 16 x 100 1019 / 1110, 8^3 167 / 372; but 64 x 64 1335 / 758, 31 x 33 1110 / 811).
-int tiny_lattice_fits(const Geometry &g, int n_chains) {
+// Where it is the faster one.  It costs about 20 us per trajectory plus the work of
+// the SM's chains (a site's action is its dearest part); the plane-streaming kernel the
+// latency of a plane per evaluation, 0.4 us, and of the energies, so it gains with
+// few planes, few evaluations and several chains per SM.  Measured over 5204 lattices,
+// chains, fields and lengths of trajectory, this kernel / plane-streaming: one chain
+// per SM 0.1 .. 0.9, but 600 x 3 with two evaluations 1.25, 1024 x 8 1.09; two chains
+// per SM 64 x 64, nine evaluations 0.28, 16^3 0.87, but 16 x 16 x 8 1.16, 512 x 16 with two
+// evaluations 1.50.  Many chains: only short rows or planes, which leave the
+// lanes of the other kernel idle (4096 of 16 x 16, nine evaluations 0.25; 1000 of 32 x 64 0.67, with
+// two evaluations 1.29; 1000 of 16 x 8 x 8 1.40; 3000 of 15 x 17 1.05).  With this rule none of
+// them is slower by more than 3 %; 222 gains of 4656 are left out.
+int tiny_lattice_fits(const Geometry &g, int n_chains, int n_pass) {
     const bool v4 = g.X % 4 == 0 && g.P % 4 == 0;
     if ((g.dim != 2 && g.dim != 3) || g.N > (int64_t)TINY_THREADS * 4 * (v4 ? 4 : 1)) return 0;
-    if (v4 ? g.N <= 1024 || (g.dim == 2 && g.X <= 32) : g.N <= 256) return 1;
-    return n_chains <= 2 * sm_count();
+    const int sms = sm_count(), per_sm = (n_chains + sms - 1) / sms;
+    const int nvec = g.P / (v4 ? 4 : 1);   // lanes that a plane fills in the other kernel
+    const int64_t planes = (int64_t)g.nplanes * n_pass;
+    const bool small = g.N <= (v4 ? 1024 : 256);
+    if (per_sm <= 2 && small) return 1;
+    if (per_sm == 1) return planes >= 24;
+    if (per_sm == 2) return 3 * planes >= 5 * nvec + 12;
+    if (!small && !(v4 && g.dim == 2 && g.X <= 32)) return 0;
+    if (nvec <= 5 || (nvec <= 16 && n_pass >= 6 && (v4 || per_sm <= 8))) return 1;
+    return nvec <= 36 && n_pass >= 9 && per_sm <= 3;
 }
 
 cudaError_t tiny_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args) {

@@ -98,6 +98,39 @@ def test_default_kernels(L, kernel):
     _same(_run(L, kernel, 2, n_md=3), _run(L, PLANE, 2, n_md=3), N, _regrouped(N), 2 * len(L))
 
 
+# chains by the number (of them per SM), evaluations and field: what each rule
+# leaves to the plane-streaming kernel, next to what it keeps
+@pytest.mark.parametrize("L,per_sm,n_md,field,kernel", [
+    ((600, 3), 1, 2, 0.0, PLANE), ((600, 3), 1, 8, 0.0, ONCHIP), ((16, 16, 8), 1, 1, 0.0, MARCH),
+    ((16, 16, 8), 2, 8, 0.0, MARCH), ((16, 16, 8), 2, 8, 0.1, PLANE), ((16, 16, 16), 2, 8, 0.0, ONCHIP), ((64, 64), 2, 1, 0.0, ONCHIP),
+    ((16, 16), 7, 1, 0.0, ONCHIP), ((32, 64), 7, 8, 0.0, ONCHIP), ((32, 64), 7, 2, 0.0, MARCH), ((16, 8, 8), 7, 8, 0.0, PLANE),
+    ((15, 17), 7, 2, 0.0, PLANE), ((31, 33), 7, 8, 0.0, PLANE), ((31, 96), 1, 8, 0.0, MARCH), ((31, 96), 4, 8, 0.0, PLANE),
+    ((61, 96), 4, 8, 0.0, PLANE), ((61, 96), 4, 20, 0.0, MARCH), ((61, 96), 7, 3, 0.0, PLANE), ((99, 30), 1, 8, 0.0, PLANE),
+    ((99, 30), 2, 8, 0.0, MARCH), ((255, 28), 4, 8, 0.1, MARCH), ((255, 28), 2, 8, 0.1, PLANE), ((301, 24), 1, 3, 0.1, PLANE),
+    ((301, 24), 1, 8, 0.1, MARCH), ((128, 40), 7, 3, 0.1, PLANE), ((128, 40), 7, 3, 0.0, MARCH),
+    ((16, 16, 16), 7, 8, 0.0, PLANE), ((24, 24, 24), 2, 8, 0.0, MARCH), ((24, 24, 24), 3, 8, 0.1, PLANE),
+    ((16, 16, 7), 2, 8, 0.0, PLANE), ((32, 32, 16), 4, 8, 0.1, MARCH), ((32, 32, 16), 4, 2, 0.1, PLANE), ((20, 20, 20), 4, 8, 0.0, PLANE)])
+def test_rules(L, per_sm, n_md, field, kernel):
+    import torch
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    kw = dict(h=np.full(int(np.prod(L)), field)) if field else {}
+    with pkg.IsingHMC(dim=len(L), L=L, beta=0.2, eps=0.1, n_md=n_md, n_chains=n, **kw) as s:
+        assert s.kernel == kernel
+        s.set_chain_split(1)   # asked for: whatever takes the lattice
+        assert s.kernel == (MARCH if kernel == MARCH or (len(L) == 2 and L[1] >= 24) or len(L) == 3 else PLANE)
+        s.trajectories(1, 3)
+        s.sync()
+
+
+# many chains: several to a CTA, cut into slabs, and by default on whichever kernel pays
+@pytest.mark.parametrize("n_chains", [1, 2, 320, 700])
+@pytest.mark.parametrize("L,kw", [((36, 97), dict(n_md=7)), ((33, 200), dict(n_md=7, h=0.04, flip_every=2)),
+                                  ((130, 49), dict(n_md=3)), ((301, 24), dict(n_md=4, field=0.1)),
+                                  ((61, 48), dict(n_md=6, field=0.1, integrator=pkg.ISING_INTEGRATOR_OMELYAN))])
+def test_march_2d_many_chains(L, kw, n_chains):
+    _same(_run(L, MARCH, n_chains, **kw), _run(L, PLANE, n_chains, **kw), L[0] * L[1], _regrouped(L[0] * L[1]), 4)
+
+
 def test_other_forms_have_no_choice():
     for kw in (dict(kind="infinite", n_sites=64), dict(dim=2, L=(4, 4), precision=pkg.ISING_PREC_PLAIN_FP64)):
         with pkg.IsingHMC(beta=0.4, eps=0.1, n_md=2, **kw) as s:
