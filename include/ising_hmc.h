@@ -31,8 +31,14 @@
  *    chain c; lattice site i = x + L0*(y + L1*z).
  *  - Philox4x32-10 (Salmon et al., SC'11) supplies every random number from a
  *    counter (index, trajectory, chain, purpose) and the key (seed lo, seed hi),
- *    so results depend only on (seed, chain, trajectory index), never on the
- *    launch shape or on how trajectories are split across calls.
+ *    so psi, p and the random numbers depend only on (seed, chain, trajectory
+ *    index), never on the launch shape, on the chains beside it or on how
+ *    trajectories are split across calls.  The sums over sites (S, H, dH,
+ *    estimators) add the same terms in an order that the kernel fixes.  On FP32
+ *    lattices the library picks the kernel and its split by the handle's number of
+ *    chains and the GPU's SMs too, so the records of a chain agree with those of
+ *    the same chain in a handle of another size, or on another GPU, to the
+ *    rounding of these sums (FP64; the estimators' per-thread parts compensated FP32).
  */
 #ifndef ISING_HMC_H
 #define ISING_HMC_H

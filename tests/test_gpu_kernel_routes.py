@@ -131,6 +131,27 @@ def test_march_2d_many_chains(L, kw, n_chains):
     _same(_run(L, MARCH, n_chains, **kw), _run(L, PLANE, n_chains, **kw), L[0] * L[1], _regrouped(L[0] * L[1]), 4)
 
 
+# the chain's own configurations and decisions do not depend on the chains beside it,
+# whichever kernel and split their number leads to
+@pytest.mark.parametrize("L", [(64, 64), (36, 96), (33, 96), (16, 16, 16), (24, 24, 24)])
+def test_chain_does_not_depend_on_its_neighbours(L):
+    N = int(np.prod(L))
+    base = 0.42 if len(L) == 2 else 0.21
+    got, kernels = [], set()
+    for n in (1, 200, 340, 1200):
+        with pkg.IsingHMC(dim=len(L), L=L, beta=base, eps=0.1, n_md=8, n_chains=n) as s:
+            kernels.add((s.kernel, n if s.kernel == MARCH else 0))
+            s.trajectories(3, 9)
+            got.append(([pkg.ising_hmc_get_chains(s.h, w, 0, 1) for w in STATES], s.records()[:1], s.chain_sums()[:1]))
+    assert len(kernels) > 1
+    for g in got[1:]:
+        for x, y in zip(g[0], got[0][0]):
+            assert np.array_equal(x, y)
+        assert np.array_equal(g[1][:, [1, 2, 7]], got[0][1][:, [1, 2, 7]])
+        assert np.abs(g[1] - got[0][1]).max() <= 1e-12 * 2 * len(L) * N
+        assert np.abs(g[2] - got[0][2])[:, :9].max() <= _regrouped(N)
+
+
 def test_other_forms_have_no_choice():
     for kw in (dict(kind="infinite", n_sites=64), dict(dim=2, L=(4, 4), precision=pkg.ISING_PREC_PLAIN_FP64)):
         with pkg.IsingHMC(beta=0.4, eps=0.1, n_md=2, **kw) as s:
