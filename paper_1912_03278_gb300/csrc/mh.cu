@@ -41,7 +41,7 @@ constexpr uint32_t PURPOSE_MH = 5;
 constexpr int MH_THREADS = 256;
 constexpr int MH_TAB = 13;   // neighbour sums -6..6
 constexpr int64_t MH_CLUSTER_WORDS = 4096;   // words per SM up to which sweeps run on clusters
-constexpr int64_t MH_WAVES_WORDS = 256;      // words per chain up to which they may take several waves
+constexpr int64_t MH_WAVES_FEW = 256, MH_WAVES_MANY = 8192;   // words per chain, see ising_mh_create
 constexpr int64_t MH_HOST_UNPACK_WORDS = 5120;
 
 // Per-chain parameters and sums.
@@ -559,9 +559,11 @@ ising_status ising_mh_create(const ising_hmc_config *cfg, ising_mh_t **out) {
     // colour's launch ends before it is under way, or where the clusters fill
     // the GPU.  Per sweep, clusters / a launch per colour: 64 chains of L = 256 8.6 /
     // 16.7 us, 300 of L = 64 5.6 / 12.3, 304 of L = 512 86 / 104; 100 of L = 512
-    // (a third of the GPU left out) 46 / 43.  More clusters than fit at once: of small
-    // chains only (twenty sweeps, per sweep: 600 of 64 x 64 7 / 14, 1000 of 128 x 128 29 / 31, of
-    // 32^3 57 / 49, of 256 x 256 92 / 87; one sweep alone 46 / 39 for 128 x 128, 85 / 57 for 32^3).
+    // (a third of the GPU left out) 46 / 43.  More clusters than fit at once: not for
+    // chains of 256 to 8192 words, whose launches per colour keep up (per sweep of
+    // many: 600 of 64 x 64 7 / 14, 4096 of 128 x 128 110 / 93, of 256 x 256 359 / 320, 1000 of 32^3 57 /
+    // 50, 1216 of 512 x 512 349 / 383, 4096 of 1024 x 1024 4453 / 6564; a sweep alone 133 / 97 for
+    // 4096 of 128 x 128).
     if (h->packed) {
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
@@ -571,7 +573,8 @@ ising_status ising_mh_create(const ising_hmc_config *cfg, ising_mh_t **out) {
             while (cs < 8 && 2 * (int64_t)cs * C <= slots && N / 32 > 64 * cs) cs *= 2;
             const int64_t ctas = (int64_t)cs * C, waves = (ctas + slots - 1) / slots;
             if ((waves == 1 && (int64_t)C * (N / 32) <= MH_CLUSTER_WORDS * (int64_t)sms) ||
-                (4 * ctas >= 3 * waves * slots && (waves == 1 || N / 32 <= MH_WAVES_WORDS)))
+                (4 * ctas >= 3 * waves * slots &&
+                 (waves == 1 || N / 32 <= MH_WAVES_FEW || N / 32 >= MH_WAVES_MANY)))
                 h->cluster = cs;
         }
         cudaGetLastError();

@@ -56,12 +56,30 @@ def test_a_launch_per_colour_in_other_dimensions(L):
     _check(L, n, [3], [7])
 
 
-# more clusters than fit at once: small chains stay on them, longer ones take a
-# launch per colour
+# more clusters than fit at once: short and long chains stay on them, those between
+# take a launch per colour
 @pytest.mark.parametrize("L,launches", [((64, 8), 1), ((128, 66), 7)])
 def test_several_waves_of_clusters(L, launches):
     import torch
     _check(L, 4 * torch.cuda.get_device_properties(0).multi_processor_count, [3], [launches])
+
+
+def test_several_waves_of_clusters_of_long_chains():
+    import torch
+    n = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    L, betas = (512, 512), np.linspace(0.3, 0.6, n)
+    sim = pkg.IsingMH(dim=2, L=L, beta=betas, n_chains=n)
+    try:
+        before = pkg.ising_mh_launch_count(sim.h)
+        sim.sweeps(2, 21)
+        assert pkg.ising_mh_launch_count(sim.h) - before == 1
+        s, sums = sim.spins(), sim.chain_sums()
+    finally:
+        sim.close()
+    for c in (0, n - 1):
+        model = oracle.Model(dim=2, L=L, beta=float(betas[c]), C=4 * float(betas[c]) + 0.1)
+        rs, rsums = oracle.mh_checkerboard(model, seed=21, chain=c, n=2)
+        assert np.array_equal(s[c], rs) and np.array_equal(sums[c], rsums), c
 
 
 # few spins are unpacked on the host, more by a launch
