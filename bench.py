@@ -171,8 +171,8 @@ def measured_peaks_all():
 
 STAGING_NAMES = {0: "auto", 1: "threads", 2: "bulk"}
 
-TRAFFIC_SOURCES = ("march_lattice.cuh", "march_lattice.cu", "pair.cuh", "df32.cuh",
-                   "device_common.cuh")
+TRAFFIC_SOURCES = ("march_lattice.cuh", "march_lattice.cu", "fused_lattice_impl.cuh", "pair.cuh",
+                   "df32.cuh", "device_common.cuh", "mbarrier.cuh", "internal.h", "device_once.h")
 
 
 def traffic_source_sha():
@@ -994,10 +994,10 @@ def mh_rate(pkg, stream, L, betas, hmc_ms, steps=4, warm=2, seed=61):
     the same chains and betas, h = 0): checkerboard Metropolis-Hastings sweeps
     timed with CUDA events, and the cost ratio T_HMC / T_MH (the paper reports
     ~4 N_step for its implementation).  L = 1024 rows take the multi-spin-
-    coded kernel, which is bound by the ALU pipe, not by HBM (0.25 B of spins
-    per site and sweep): its roofline is the ALU-pipe saturation rate; the
-    HBM fraction at 2 B per site-sweep (int8 spins) is kept for comparison
-    with the byte kernels."""
+    coded form, whole sweeps on a cluster of CTAs per chain, which is bound by the
+    ALU pipe, not by HBM (0.25 B of spins per site and sweep): its roofline is
+    the ALU-pipe saturation rate; the HBM fraction at 2 B per site-sweep (int8
+    spins) is kept for comparison with the byte kernels."""
     import torch
     n = len(betas)
     sim = pkg.IsingMH(dim=2, L=(L, L), beta=betas, n_chains=n, stream=stream.cuda_stream)
@@ -1018,11 +1018,11 @@ def mh_rate(pkg, stream, L, betas, hmc_ms, steps=4, warm=2, seed=61):
     sites = float(L) * L * n
     peak, peak_kind = measured_peaks()
     achieved = 2.0 * sites / (ms / 1e3) / 1e9
-    # the packed kernel is bound by the ALU pipe (Philox and bit logic): peak =
-    # the decision rate at which that pipe would be saturated, from the ncu
-    # capture of one colour launch of 2048 chains at L = 1024 (1.0737e9
-    # decisions in 1.564 ms with the ALU pipe 68.86% busy)
-    alu_peak = 1.0737e9 / 1.564e-3 / 0.6886
+    # bound by the ALU pipe (Philox and bit logic): peak = the decision rate at which
+    # that pipe would be saturated, from the ncu capture of two sweeps of 608
+    # chains at L = 1024 (1.2751e9 decisions in 1.3359 ms with the ALU pipe 64.17%
+    # busy, 25.3 thread instructions per decision)
+    alu_peak = 1.2751e9 / 1.3359e-3 / 0.6417
     return {"workload": "2D L=%d, %d chains (16 betas in [0.38, 0.50]), J=1, h=0, checkerboard, "
                         "spins start +1, %d warm-up sweeps" % (L, n, warm),
             "value": sites / (ms / 1e3), "unit": "site-updates/s", "ms_per_sweep": ms,
@@ -1032,7 +1032,7 @@ def mh_rate(pkg, stream, L, betas, hmc_ms, steps=4, warm=2, seed=61):
                          "unit": "site-updates/s", "frac": sites / (ms / 1e3) / alu_peak,
                          "peak_source": "derived: ALU-pipe saturation rate from the ncu counters "
                                         "(profiles/mh_packed_kernel_2d_L1024.md)",
-                         "kernel": "mh_packed_kernel (both colours + measurement)",
+                         "kernel": "mh_cluster_kernel (whole sweeps)",
                          "hbm_fraction_at_2_bytes_per_site_sweep": achieved / peak}}
 
 
