@@ -29,7 +29,8 @@
 // (pair.cuh: the scalar operations' bits): the resident kernel is bound by issue
 // (2432 chains of N = 4096: 0.50 -> 0.47 ms per call of one trajectory), the streaming
 // one by issue and latency (304 chains of N = 50001: 1.35 -> 1.14 ms; with kept
-// quads 1.00, with batched loads 0.78).
+// quads 1.00, with batched loads 0.78).  128 registers at most (two CTAs of 256 threads on an SM);
+// only the resident instances of eight quads a thread spill, 544 .. 648 bytes (stores).
 #include <cuda_runtime.h>
 
 #include "df32.cuh"

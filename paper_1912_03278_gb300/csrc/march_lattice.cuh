@@ -34,6 +34,13 @@
 // A chain whose rows fill only part of a CTA can be cut into slabs of rows, one
 // per group of threads (few chains, which would leave the SMs without warps).
 //
+// Registers: 128 a thread (two CTAs of 256 threads on an SM) are fewer than the three
+// evaluations want.  The compiler spills 116 .. 144 bytes a thread (stores; loads 156 ..
+// 256) for rows of whole vectors, 320 .. 404 (448 .. 588) with a field per site, and for
+// ragged rows, whose draws and masks come on top, 1204 .. 1368 (1640 .. 1856), with a
+// field 1808 .. 1820 (1884 .. 1924): the reason that march_lattice_pays leaves many of
+// those to the plane-streaming kernel.
+//
 // Every value is computed by the operations of the plane-streaming kernel in
 // the same order (the packed FP32 pair instructions round each half exactly as
 // the scalar ones do): psi and p agree bit for bit, and so do the per-thread
@@ -735,7 +742,9 @@ __global__ void __launch_bounds__(MARCH_CTA_THREADS, 2)
 // of the action): several chains each as long as that leaves two CTAs for every
 // SM; fewer chains than that are cut into slabs instead, as long as the slabs
 // have rows enough (12 rows more than its own are computed per slab and sweep)
-// and the SMs room for them.  L = 251 x 173, 304 chains, minimum-norm integrator
+// and the SMs threads for them.  (Not for their shared memory: eight slabs of one warp take 117
+// KB, each with a reduction block of which the chain uses one, so a single CTA of them
+// fits on an SM and more chains than SMs take two turns.)  L = 251 x 173, 304 chains, minimum-norm integrator
 // of 6 steps: 1.93 ms uncut (four warps per SM), 0.97 ms in four slabs; 64 chains
 // of L = 128, N_md = 20: 0.18 ms in four slabs (1.53 ms on the plane-streaming
 // kernel).

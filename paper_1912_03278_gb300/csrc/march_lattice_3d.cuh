@@ -14,6 +14,14 @@
 //
 // psi and p are computed by the operations of the plane-streaming kernel in
 // the same order and agree bit for bit.
+//
+// What bounds it: HBM where the planes of all chains do not stay in L2 (152 chains of
+// 64^3: 6.5 TB/s in the middle evaluations); else the latency of one plane after
+// the other at four to sixteen warps per SM (64 chains of 32^3 on four CTAs each: 147 us per
+// trajectory of 11 evaluations, issue 33 %, DRAM 1 %, stalls wait 1.3, long
+// scoreboard 0.6, barrier 0.5 per issue).  128 registers; spills 336 .. 452 bytes a
+// thread (stores; loads 344 .. 616), with a field 512 .. 604 (528 .. 728), in the first and
+// last evaluations' draws and action.
 #pragma once
 #include "march_lattice.cuh"
 

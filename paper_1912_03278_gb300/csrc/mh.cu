@@ -554,8 +554,8 @@ ising_status ising_mh_create(const ising_hmc_config *cfg, ising_mh_t **out) {
             return bail(mh_fail(h, ISING_ECUDA, "stream creation failed"));
         h->own_stream = true;
     }
-    // Whole sweeps on a cluster per chain (up to eight CTAs, as many as two of
-    // 1024 threads per SM allow): where the words of all chains are few, so that a
+    // Whole sweeps on a cluster per chain, up to eight CTAs, as many as make two per SM
+    // (at 42 registers two of up to 672 threads are resident, of 1024 one): where the words of all chains are few, so that a
     // colour's launch ends before it is under way, or where the clusters fill
     // the GPU.  Per sweep, clusters / a launch per colour: 64 chains of L = 256 8.6 /
     // 16.7 us, 300 of L = 64 5.6 / 12.3, 304 of L = 512 86 / 104; 100 of L = 512

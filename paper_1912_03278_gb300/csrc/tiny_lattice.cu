@@ -6,7 +6,9 @@
 // each).  Here all sites are updated at once, two barriers per evaluation; HBM is
 // touched once per trajectory (the proposal and the end momenta, which stay
 // readable).  64 chains of 16 x 16, N_md = 5, eight trajectories: 0.09 ms, on the
-// plane-streaming kernel 0.71.
+// plane-streaming kernel 0.71.  Latency bounds it: two warps on each of 64 SMs, issue 14 % of
+// the cycles, stalls per issue wait 2.9, barrier 1.2, short scoreboard 1.0, no instruction
+// 0.9; 117 registers, no spills.
 //
 // psi and p are computed by its operations in the same order and agree bit for
 // bit.  So do the estimators' compensated FP32 sums: Kahan's scheme rounds every
