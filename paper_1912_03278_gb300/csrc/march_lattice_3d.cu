@@ -38,22 +38,30 @@ int march3_lattice_split(const Geometry &g, int n_chains) {
 
 // Planes of few tiles leave its CTAs with one or two warps and few of those fit on an
 // SM, so many such chains, and a field's loads, which nothing hides, are the
-// plane-streaming kernel's.  Against its time, nine evaluations (with a field per site):
-// 152 chains of 24^3 0.71 (0.89), 304 of 20^3 0.89 (1.00), of 24^3 0.91 (1.11), of 32^3 0.82 (0.98), 1000 of
-// 16^3 1.18 (1.54), of 12^3 0.90 (1.10), of 8 x 8 x 20 1.11 (1.30), of 20^3 0.97 (1.23), of 28^3 0.82
+// plane-streaming kernel's; where all CTAs are resident at once it holds its own.  Against
+// that kernel's time, nine evaluations (with a field per site): 152 chains of 24^3 0.71 (0.89),
+// 304 of 20^3 0.89 (1.00), of 24^3 0.91 (1.11), of 32^3 0.82 (0.98), 608 of 20^3 0.87 (1.10), of 16^3 0.94
+// (1.13), 1000 of 16^3 (912 fit) 1.18 (1.54), of 12^3 0.90 (1.10), of 8 x 8 x 20 1.11 (1.30), of 28^3 0.82
 // (1.05), of 32 x 32 x 16 0.65 (0.87); two evaluations, 304 of 24^3 1.11 (1.30).  Of fewer than
-// eight planes the four extra ones of every evaluation eat the gain (348 drawn lattices
-// 0.96 in the mean, a third of them slower).  With this rule one of 1750 lattices is
-// slower by more than 3 % (by 4).
+// eight planes the four extra ones of every evaluation eat the gain but for full, large
+// planes (389 of 32 x 56 x 7 0.73).  With this rule 11 of 2402 lattices are slower by more than
+// 3 % (the worst 1.25, with a sign flip per trajectory); 206 gains of 1662 are left out.
 int march3_lattice_pays(const Geometry &g, int n_chains, int n_pass, bool field) {
     const int T = m3_threads(g.X, g.Y), tiles = (g.X / 4) * ((g.Y + 1) / 2);
     const int sms = sm_count(), per_sm = (n_chains + sms - 1) / sms, cs = march3_lattice_split(g, n_chains);
-    const bool longer = n_pass >= 9;
-    if (g.nplanes < 8) return 0;
+    const bool longer = n_pass >= 8, full = 8 * tiles >= 7 * T;
+    if (g.nplanes < 8) return g.nplanes >= 6 && !field && T >= 128 && longer && full;
     if (T >= 256 || cs >= 4) return 1;
-    if (!field) return T >= 128 || per_sm == 1 || (longer && (T >= 96 || per_sm <= 3 || (T == 64 && tiles == T)));
-    if (T >= 128) return (per_sm == 1 && (longer || T >= 192)) || (longer && 8 * tiles >= 7 * T);
-    return longer && cs >= 2 && per_sm <= 2 && (T >= 64 || g.nplanes >= 16);
+    if (field) {
+        if (T >= 128) return (per_sm == 1 && (longer || T >= 192)) || (longer && full);
+        return longer && cs >= 2 && per_sm <= 2 && (T >= 64 || g.nplanes >= 16);
+    }
+    if (T >= 128 || per_sm == 1) return 1;
+    if (n_pass < 5) return 0;
+    if (T >= 96) return longer || cs >= 2 || full;
+    if (per_sm <= 2) return longer || cs >= 2;
+    return longer && (per_sm <= 3 || (per_sm == 4 && g.nplanes >= 20) || (T == 64 && tiles == T) ||
+                      (tiles >= 18 && n_chains <= sms * march3_resident(g)));
 }
 
 cudaError_t march3_lattice_node(const FusedArgs &a, cudaKernelNodeParams *np, void **args) {

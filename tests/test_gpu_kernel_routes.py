@@ -105,11 +105,12 @@ def test_default_kernels(L, kernel):
     ((16, 16, 8), 2, 8, 0.0, MARCH), ((16, 16, 8), 2, 8, 0.1, PLANE), ((16, 16, 16), 2, 8, 0.0, ONCHIP), ((64, 64), 2, 1, 0.0, ONCHIP),
     ((16, 16), 7, 1, 0.0, ONCHIP), ((32, 64), 7, 8, 0.0, ONCHIP), ((32, 64), 7, 2, 0.0, MARCH), ((16, 8, 8), 7, 8, 0.0, PLANE),
     ((15, 17), 7, 2, 0.0, PLANE), ((31, 33), 7, 8, 0.0, PLANE), ((31, 96), 1, 8, 0.0, MARCH), ((31, 96), 4, 8, 0.0, PLANE),
-    ((61, 96), 4, 8, 0.0, PLANE), ((61, 96), 4, 20, 0.0, MARCH), ((61, 96), 7, 3, 0.0, PLANE), ((99, 30), 1, 8, 0.0, PLANE),
-    ((99, 30), 2, 8, 0.0, MARCH), ((255, 28), 4, 8, 0.1, MARCH), ((255, 28), 2, 8, 0.1, PLANE), ((301, 24), 1, 3, 0.1, PLANE),
+    ((61, 96), 4, 8, 0.0, MARCH), ((61, 96), 4, 8, 0.1, PLANE), ((61, 96), 7, 20, 0.0, MARCH), ((61, 96), 7, 3, 0.0, PLANE), ((99, 30), 1, 8, 0.0, PLANE),
+    ((99, 30), 2, 8, 0.0, MARCH), ((255, 28), 4, 8, 0.1, MARCH), ((255, 28), 2, 8, 0.1, PLANE), ((255, 28), 8, 3, 0.1, MARCH), ((255, 28), 7, 3, 0.1, PLANE), ((301, 24), 1, 3, 0.1, PLANE),
     ((301, 24), 1, 8, 0.1, MARCH), ((128, 40), 7, 3, 0.1, PLANE), ((128, 40), 7, 3, 0.0, MARCH),
     ((16, 16, 16), 7, 8, 0.0, PLANE), ((24, 24, 24), 2, 8, 0.0, MARCH), ((24, 24, 24), 3, 8, 0.1, PLANE),
-    ((16, 16, 7), 2, 8, 0.0, PLANE), ((32, 32, 16), 4, 8, 0.1, MARCH), ((32, 32, 16), 4, 2, 0.1, PLANE), ((20, 20, 20), 4, 8, 0.0, PLANE)])
+    ((16, 16, 7), 2, 8, 0.0, PLANE), ((32, 32, 16), 4, 8, 0.1, MARCH), ((32, 32, 16), 4, 2, 0.1, PLANE), ((20, 20, 20), 4, 8, 0.0, MARCH), ((20, 20, 20), 6, 8, 0.0, PLANE),
+    ((32, 56, 7), 3, 8, 0.0, MARCH), ((31, 96), 3, 8, 0.0, MARCH), ((31, 96), 4, 30, 0.0, MARCH), ((31, 96), 4, 20, 0.1, PLANE)])
 def test_rules(L, per_sm, n_md, field, kernel):
     import torch
     n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
@@ -120,6 +121,14 @@ def test_rules(L, per_sm, n_md, field, kernel):
         assert s.kernel == (MARCH if kernel == MARCH or (len(L) == 2 and L[1] >= 24) or len(L) == 3 else PLANE)
         s.trajectories(1, 3)
         s.sync()
+
+
+def test_sign_flips_count_as_shorter_trajectories():
+    import torch
+    n = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    for flip, kernel in ((0, MARCH), (1, PLANE), (4, MARCH)):
+        with pkg.IsingHMC(dim=3, L=(24, 24, 24), beta=0.2, eps=0.1, n_md=8, n_chains=n, flip_every=flip) as s:
+            assert s.kernel == kernel
 
 
 # many chains: several to a CTA, cut into slabs, and by default on whichever kernel pays
