@@ -22,7 +22,7 @@ int march_lattice_threads(const Geometry &g) {
 // (1.45), 255 x 24 0.92 (1.17), 301 x 24 0.68 (0.85); 608 of 61 x 64 0.87 (1.03), 1000 of 31 x 64
 // 1.41 (1.73), of 61 x 64 1.04 (1.30), of 99 x 64 0.61 (0.80), of 255 x 28 0.50 (0.76); two
 // evaluations, 1000 of 61 x 60 1.82 (1.88), 21: 1000 of 61 x 60 0.79 (1.08).  With this rule one of
-// 5961 is slower by more than 3 % (by 3.5); 552 gains of 3802 are left out.
+// 5961 is slower by more than 3 % (by 3.5); 548 gains of 3802 are left out.
 int march_lattice_pays(const Geometry &g, int n_chains, int n_pass, bool field) {
     const int sms = sm_count(), per_sm = (n_chains + sms - 1) / sms;
     if (g.X % 4 == 0) return !(field && n_pass <= 4 && per_sm >= 5);

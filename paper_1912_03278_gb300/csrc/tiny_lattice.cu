@@ -287,7 +287,7 @@ cudaError_t tiny_qpt(const FusedArgs &a, cudaKernelNodeParams *np, void **args) 
 // evaluations 1.50.  Many chains: only short rows or planes, which leave the
 // lanes of the other kernel idle (4096 of 16 x 16, nine evaluations 0.25; 1000 of 32 x 64 0.67, with
 // two evaluations 1.29; 1000 of 16 x 8 x 8 1.40; 3000 of 15 x 17 1.05).  With this rule none of
-// them is slower by more than 3 %; 222 gains of 4656 are left out.
+// them is slower by more than 3 %; 234 gains of 4656 are left out.
 int tiny_lattice_fits(const Geometry &g, int n_chains, int n_pass) {
     const bool v4 = g.X % 4 == 0 && g.P % 4 == 0;
     if ((g.dim != 2 && g.dim != 3) || g.N > (int64_t)TINY_THREADS * 4 * (v4 ? 4 : 1)) return 0;

@@ -92,3 +92,24 @@ def test_spins_are_read_back_under_a_busy_default_stream(L):
         assert np.array_equal(s.spins(), spins)
     finally:
         s.close()
+
+
+def test_native_copies_under_capture_are_refused_and_leave_the_capture_usable():
+    import torch
+    st = torch.cuda.Stream()
+    kw = dict(KINDS["lattice"], stream=st.cuda_stream)
+    with pkg.IsingHMC(**kw) as a, pkg.IsingHMC(**kw) as b:
+        buf = torch.zeros(a.state().shape, device="cuda")
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            for call in (lambda: pkg.ising_hmc_set_state_native(a.h, buf.data_ptr(), 0),
+                         lambda: pkg.ising_hmc_get_state_native(a.h, buf.data_ptr())):
+                with pytest.raises(pkg.IsingError):
+                    call()
+            a.trajectories(2, 7)
+        with torch.cuda.stream(st):
+            g.replay()
+        b.trajectories(2, 7)
+        torch.cuda.synchronize()
+        assert np.array_equal(a.state(), b.state())
